@@ -9,105 +9,169 @@
 // norm (the delta rule's keys); q and v are not.  The outputs are rounded to
 // bf16, the delta rule's operand type.
 //
-// grid.x < sum M: one block per (tail token, head) computes y for its head's
-// q, k and v channels; grid.x >= sum M: one block per (character, head)
-// writes the character's new state (the last three inputs of [state; tail])
-// into the other of two state buffers, so that no block reads a state row
-// that another block of the same launch writes.
+// Bound by memory: every input is read and every output written once.  A
+// thread owns eight channels (16 bytes of a token's row) and walks a strip of
+// consecutive packed tokens with the taps and the last three inputs in
+// registers, four rows in flight; a head's d_k / 8 neighbouring lanes share
+// the norm of k.  Strips are as long as the grid allows: a strip's first
+// three rows are read again.
+//
+// blockIdx.y < n_strips: outputs of a strip; beyond: one row of blocks per
+// character writes the character's new state (the last three inputs of
+// [state; tail]) into the other of two state buffers, so that no block reads
+// a state row that another block of the same launch writes.
 #include "kvm_internal.cuh"
 
 namespace kvm {
 namespace {
 
-__device__ __forceinline__ float silu(float x) { return x / (1.f + __expf(-x)); }
+constexpr int kThreads = 128;
+constexpr int kAhead = 4;                    // rows loaded ahead of their use
 
-// First channel of the k part (q channels come first, then k, then v).
-__device__ __forceinline__ int H_off_k(const ConvParams& p) { return p.H * p.dk; }
+// the quotient to 2 ulp (the result is rounded to bf16)
+__device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.f + __expf(-x)); }
 
-__global__ void __launch_bounds__(128) gdn_conv_kernel(const __grid_constant__ ConvParams p) {
+using f2 = unsigned long long;               // two packed floats
+
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Eight bf16 channels as four pairs of floats.
+__device__ __forceinline__ void unpack8(const uint4& v, f2* x) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(&v);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]));
+        x[e] = pack2(f.x, f.y);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 4) gdn_conv_kernel(const __grid_constant__ ConvParams p) {
+    const int g = blockIdx.x * kThreads + threadIdx.x;       // channels 8 g .. 8 g + 7
+    const bool act = 8 * g < p.channels;
+    const int hk = p.H * p.dk, c = act ? 8 * g : 0;
+    const bool is_k = act && c >= hk && c < 2 * hk;
+    // the part's rows are contiguous: [tok][H d_k] or [tok][H d_v]
+    const int first = c < hk ? 0 : c < 2 * hk ? hk : 2 * hk;
+    const int64_t stride = c < 2 * hk ? hk : p.H * p.dv;
+    const __nv_bfloat16* in = (c < hk ? p.xq : c < 2 * hk ? p.xk : p.xv) + (c - first);
+    __nv_bfloat16* out = (c < hk ? p.yq : c < 2 * hk ? p.yk : p.yv) + (c - first);
+    auto row = [&](int64_t tok) { return *reinterpret_cast<const uint4*>(in + tok * stride); };
+    auto old_row = [&](int b, int r) {
+        return *reinterpret_cast<const uint4*>(p.state_in + ((int64_t)b * 3 + r) * p.channels + c);
+    };
     grid_dependency_wait();
     grid_dependents_launch();
-    const int h = blockIdx.y;
-    const int dk = p.dk, dv = p.dv, C = p.channels;
-    const int per_head = 2 * dk + dv;
-    if ((int)blockIdx.x >= p.total) {
-        // new conv state of one character's channels of head h
-        const int b = blockIdx.x - p.total;
+    if ((int)blockIdx.y >= p.n_strips) {
+        const int b = blockIdx.y - p.n_strips;
         if (b >= p.n_chars) { if (threadIdx.x == 0) atomicOr(p.err, kErrBounds); return; }
+        if (!act) return;
         const int M = p.tail_cu[b + 1] - p.tail_cu[b];
-        const __nv_bfloat16* old_s = p.state_in + (int64_t)b * 3 * C;
-        __nv_bfloat16* new_s = p.state_out + (int64_t)b * 3 * C;
-        for (int e = threadIdx.x; e < 3 * per_head; e += blockDim.x) {
-            const int r = e / per_head, j = e % per_head;
-            // channel of element j of this head
-            const int c = j < dk ? h * dk + j
-                        : j < 2 * dk ? H_off_k(p) + h * dk + (j - dk) : 2 * H_off_k(p) + h * dv + (j - 2 * dk);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
             const int t = M - 3 + r;                         // position in the tail (negative: old state row t + 3)
-            __nv_bfloat16 x;
-            if (t >= 0) {
-                const int64_t tok = p.tail_cu[b] + t;
-                x = j < dk ? p.xq[(tok * p.H + h) * dk + j]
-                  : j < 2 * dk ? p.xk[(tok * p.H + h) * dk + (j - dk)]
-                               : p.xv[(tok * p.H + h) * dv + (j - 2 * dk)];
-            } else {
-                x = old_s[(int64_t)(t + 3) * C + c];
-            }
-            new_s[(int64_t)r * C + c] = x;
+            *reinterpret_cast<uint4*>(p.state_out + ((int64_t)b * 3 + r) * p.channels + c) =
+                t >= 0 ? row(p.tail_cu[b] + t) : old_row(b, t + 3);
         }
         return;
     }
-    const int n = blockIdx.x;                                // packed tail token
-    int lo = 0, hi = p.n_chars - 1;                          // last b with tail_cu[b] <= n
+    const int n0 = blockIdx.y * p.strip, n1 = min(p.total, n0 + p.strip);
+    int lo = 0, hi = p.n_chars - 1;                          // last b with tail_cu[b] <= n0
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (p.tail_cu[mid] <= n) lo = mid; else hi = mid - 1;
+        if (p.tail_cu[mid] <= n0) lo = mid; else hi = mid - 1;
     }
-    const int b = lo;
-    const int t = n - p.tail_cu[b];
-    const __nv_bfloat16* old_s = p.state_in + (int64_t)b * 3 * C;
-    __shared__ float ksq[4];
-    float kval = 0.f;                                        // d_k <= 128 threads: at most one k channel each
-    float part = 0.f;
-    for (int j = threadIdx.x; j < per_head; j += blockDim.x) {
-        const bool is_q = j < dk, is_k = !is_q && j < 2 * dk;
-        const int jj = is_q ? j : is_k ? j - dk : j - 2 * dk;
-        const int c = is_q ? h * dk + jj : is_k ? H_off_k(p) + h * dk + jj : 2 * H_off_k(p) + h * dv + jj;
-        const __nv_bfloat16* src = is_q ? p.xq : is_k ? p.xk : p.xv;
-        const int width = (is_q || is_k) ? dk : dv;
-        float acc = 0.f;
+    int b = lo, end = p.tail_cu[b + 1];
+    f2 w[4][4];                                              // [tap][channel pair]
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int tt = t - 3 + i;                         // input row of tap i
-            float x;
-            if (tt >= 0) x = __bfloat162float(src[((int64_t)(p.tail_cu[b] + tt) * p.H + h) * width + jj]);
-            else x = __bfloat162float(old_s[(int64_t)(tt + 3) * C + c]);
-            acc = fmaf(p.w[(int64_t)c * 4 + i], x, acc);
+    for (int e = 0; e < 4; ++e) {
+        const float4 f = *(reinterpret_cast<const float4*>(p.w) + c + 2 * e);
+        const float4 g = *(reinterpret_cast<const float4*>(p.w) + c + 2 * e + 1);
+        w[0][e] = pack2(f.x, g.x); w[1][e] = pack2(f.y, g.y); w[2][e] = pack2(f.z, g.z); w[3][e] = pack2(f.w, g.w);
+    }
+    f2 x[4][4];                                              // the inputs of taps 0 .. 3
+    // the three inputs before token n of character b
+    auto history = [&](int n) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int t = n - p.tail_cu[b] - 3 + i;
+            unpack8(t >= 0 ? row(n - 3 + i) : old_row(b, t + 3), x[i]);
         }
-        const float y = silu(acc);
-        if (is_k) {
-            kval = y;                                         // normalised below
-            part = fmaf(y, y, part);
-        } else {
-            __nv_bfloat16* dst = is_q ? p.yq : p.yv;
-            dst[((int64_t)n * p.H + h) * width + jj] = __float2bfloat16_rn(y);
+    };
+    const bool any_k = __any_sync(0xffffffffu, is_k);
+    uint4 next[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) next[u] = n0 + u < n1 ? row(n0 + u) : make_uint4(0, 0, 0, 0);
+    history(n0);
+    for (int n = n0; n < n1; n += kAhead) {
+        uint4 now[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            now[u] = next[u];
+            if (n + kAhead + u < n1) next[u] = row(n + kAhead + u);
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            if (n + u >= n1) break;                          // uniform per block
+            if (n + u == end) {                              // the next character with a tail
+                do ++b; while (p.tail_cu[b + 1] == p.tail_cu[b]);
+                end = p.tail_cu[b + 1];
+                history(n + u);
+            }
+            unpack8(now[u], x[3]);
+            float y[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                f2 acc = 0;                                  // two zeros
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc = fma2(w[i][e], x[i][e], acc);
+                const float2 a = unpack2(acc);
+                y[2 * e] = silu(a.x);
+                y[2 * e + 1] = silu(a.y);
+            }
+            if (any_k) {                                     // uniform per warp
+                float tot = 0.f;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) tot = fmaf(y[e], y[e], tot);
+                for (int o = p.dk / 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+                if (is_k) {
+                    const float inv = tot > 0.f ? rsqrtf(tot) : 0.f;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) y[e] *= inv;
+                }
+            }
+            uint4 o4;
+            __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&o4);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o2[e] = __floats2bfloat162_rn(y[2 * e], y[2 * e + 1]);
+            if (act) *reinterpret_cast<uint4*>(out + (int64_t)(n + u) * stride) = o4;
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[i][e] = x[i + 1][e];
         }
     }
-    // ||k||^2 over the head: warp sums, then the block's four warps
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if ((threadIdx.x & 31) == 0) ksq[threadIdx.x >> 5] = part;
-    __syncthreads();
-    const float norm2 = ksq[0] + ksq[1] + ksq[2] + ksq[3];
-    const float inv = norm2 > 0.f ? rsqrtf(norm2) : 0.f;
-    for (int j = threadIdx.x; j < per_head; j += blockDim.x)
-        if (j >= dk && j < 2 * dk) p.yk[((int64_t)n * p.H + h) * dk + (j - dk)] = __float2bfloat16_rn(kval * inv);
 }
 
 }  // namespace
 
 void launch_gdn_conv(const ConvParams& p, cudaStream_t s) {
     if (p.total <= 0) return;
-    launch_pdl(gdn_conv_kernel, dim3(p.total + p.n_chars, p.H), dim3(128), 0, s, p);
+    launch_pdl(gdn_conv_kernel, dim3((p.channels / 8 + kThreads - 1) / kThreads, p.n_strips + p.n_chars), dim3(kThreads),
+               0, s, p);
 }
 
 }  // namespace kvm

@@ -1127,6 +1127,11 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         cp.n_chars = c->B;
         cp.H = c->H; cp.dk = c->dk; cp.dv = c->dv; cp.channels = c->conv_ch;
         cp.total = total;
+        // strips of up to 32 tokens while the threads (one per eight channels
+        // and strip) fill the SMs, at least 4
+        cp.strip = 32;
+        while (cp.strip > 4 && (int64_t)total * (c->conv_ch / 8) / cp.strip < 1024 * (int64_t)c->num_sms) cp.strip /= 2;
+        cp.n_strips = (total + cp.strip - 1) / cp.strip;
         for (int b = 0; b <= c->B; ++b) cp.tail_cu[b] = tail_cu[b];
         cp.xq = p.q; cp.xk = p.k; cp.xv = p.v;
         cp.w = c->conv_w + (size_t)g * c->conv_ch * 4;

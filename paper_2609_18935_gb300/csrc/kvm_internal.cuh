@@ -245,6 +245,7 @@ struct GdnParams {
 struct ConvParams {
     int32_t n_chars, H, dk, dv, channels;     // channels = H (2 d_k + d_v)
     int32_t total;                            // sum M
+    int32_t strip, n_strips;                  // packed tokens a thread walks; ceil(total / strip)
     int32_t tail_cu[kMaxChars + 1];
     const __nv_bfloat16* xq;                  // caller's pre-conv inputs [sum M][H][d_k]
     const __nv_bfloat16* xk;
