@@ -59,6 +59,13 @@ int attention_grid_cap(int num_sms, int head_dim) {
 constexpr int kMinUnitsPerCta = 4;  // smallest share of (query tile, key tile) units per attention block
 constexpr double kSegmentCost = 8.0; // extra cost, in 64-key units, of each segment an attention block starts
 constexpr int kFlagStride = 32;     // compaction read flags: one per 128-byte line
+// Longest tail of the token-by-token delta rule, by d_k.  Measured against the
+// chunked form (back-to-back layers, d_v = d_k, us): at d_k 128, 16 heads, 32
+// tokens 9.5 against 14.0 for one character, 21 : 24 for 8, 60 : 90 for 32, but
+// 40 tokens 26 : 24 for 8; at d_k 64, 48 tokens 11 : 13, 16 : 18, 35 : 63, but 64
+// tokens 14 : 12.7 and 21 : 18 for 1 and 8.
+constexpr int recur_tail(int dk) { return dk == 64 ? 48 : 32; }
+constexpr int kRecurTile = 16;      // tokens it stages at a time when blocks share an SM
 constexpr int kMinPrepWorkers = 24; // fused delta-rule launches leave at least this many SMs to the prep
 
 }  // namespace
@@ -1091,6 +1098,17 @@ kvm_status do_attention(kvm_ctx* c, int layer, const int32_t* tail_cu, const voi
     return KVM_OK;
 }
 
+// Rows of S per eight lanes of the token-by-token delta rule: four (k and q
+// read from shared memory once for four rows) while that leaves about a block
+// an SM, else fewer, for more SMs and a shorter step.  16 tokens, 16 heads of
+// 128, with 1 | 2 | 4 rows: one character 5.6 | 6.6 | 8.1 us, 8 characters
+// 17.7 | 12.3 | 11.8, 32 characters 49 | 35 | 32.
+int recur_rows(const kvm_ctx* c, int active) {
+    int nr = c->dv % 64 == 0 ? 4 : 2;
+    while (nr > 1 && 4 * (int64_t)active * c->H * (c->dv / (16 * nr)) < 3 * c->num_sms) nr /= 2;
+    return nr;
+}
+
 kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, const void* k, const void* v,
                   const float* alpha, const float* beta, void* out, cudaStream_t s) {
     kvm_status st = check_layer(c, layer, KVM_LAYER_GDN);
@@ -1100,25 +1118,18 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     if (st) return st;
     if (total == 0) return KVM_OK;
     if (!q || !k || !v || !alpha || !beta || !out) return fail(KVM_E_INVAL, "NULL tensor");
-    thread_local static GdnParams p;
-    std::memset(&p, 0, sizeof p);
-    p.n_chars = c->B;
-    p.H = c->H; p.dk = c->dk; p.dv = c->dv;
-    // d_v rows of a head's state per scan block: split the rows (down to 32)
-    // until the (character, head, slice) blocks cover the SMs
-    {
-        int active = 0;
-        for (int b = 0; b < c->B; ++b) active += (tail_cu[b + 1] > tail_cu[b]);
-        int slices = 1;
-        while (c->dv / (2 * slices) >= 32 && c->dv % (2 * slices * 32) == 0 &&
-               (int64_t)active * c->H * slices < c->num_sms)
-            slices *= 2;
-        p.dv_slice = c->dv / slices;
+    int active = 0, longest = 0;
+    for (int b = 0; b < c->B; ++b) {
+        const int m = tail_cu[b + 1] - tail_cu[b];
+        active += m > 0;
+        longest = std::max(longest, m);
     }
-    p.q = static_cast<const __nv_bfloat16*>(q);
-    p.k = static_cast<const __nv_bfloat16*>(k);
-    p.v = static_cast<const __nv_bfloat16*>(v);
-    if (c->conv) {
+    const bool recur = longest <= recur_tail(c->dk) && !c->gdn_chain;
+    // its blocks each convolve their head's q and k themselves: cheaper than a
+    // launch for a few tokens (one character's decode step 4.0 against 4.4 us,
+    // 32 characters' 15.6 against 16.4; at 4 tokens 6.4 : 7.5 and 25 : 21)
+    const bool conv_inside = c->conv && recur && (longest <= 2 || (longest <= 4 && total <= 32));
+    if (c->conv && !conv_inside) {
         // short convolution + SiLU (+ k normalisation) from the carried conv
         // state; the delta rule then reads the convolved q, k, v
         thread_local static ConvParams cp;
@@ -1133,7 +1144,9 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         while (cp.strip > 4 && (int64_t)total * (c->conv_ch / 8) / cp.strip < 1024 * (int64_t)c->num_sms) cp.strip /= 2;
         cp.n_strips = (total + cp.strip - 1) / cp.strip;
         for (int b = 0; b <= c->B; ++b) cp.tail_cu[b] = tail_cu[b];
-        cp.xq = p.q; cp.xk = p.k; cp.xv = p.v;
+        cp.xq = static_cast<const __nv_bfloat16*>(q);
+        cp.xk = static_cast<const __nv_bfloat16*>(k);
+        cp.xv = static_cast<const __nv_bfloat16*>(v);
         cp.w = c->conv_w + (size_t)g * c->conv_ch * 4;
         cp.state_in = conv_state_of(c, g, c->conv_par[g]);
         cp.state_out = conv_state_of(c, g, c->conv_par[g] ^ 1);
@@ -1146,8 +1159,54 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         prof_end(c, ps, s);
         LAUNCH_CHECK(c);
         c->conv_par[g] ^= 1;
-        p.q = cp.yq; p.k = cp.yk; p.v = cp.yv;
+        q = cp.yq; k = cp.yk; v = cp.yv;
     }
+    if (recur) {
+        // token by token in one launch
+        thread_local static RecurParams rp;
+        std::memset(&rp, 0, sizeof rp);
+        const int g = c->gdn_idx[layer];
+        rp.n_chars = c->B;
+        rp.H = c->H; rp.dk = c->dk; rp.dv = c->dv; rp.channels = c->conv_ch;
+        std::copy(tail_cu, tail_cu + c->B + 1, rp.tail_cu);
+        rp.q = static_cast<const __nv_bfloat16*>(q);
+        rp.k = static_cast<const __nv_bfloat16*>(k);
+        rp.v = static_cast<const __nv_bfloat16*>(v);
+        rp.alpha = alpha;
+        rp.beta = beta;
+        rp.out = static_cast<__nv_bfloat16*>(out);
+        rp.S = c->S + (size_t)g * c->B * c->H * c->dv * c->dk;
+        if (conv_inside) {
+            rp.w = c->conv_w + (size_t)g * c->conv_ch * 4;
+            rp.state_in = conv_state_of(c, g, c->conv_par[g]);
+            rp.state_out = conv_state_of(c, g, c->conv_par[g] ^ 1);
+        }
+        const int nr = recur_rows(c, active);
+        const bool few = (int64_t)active * c->H * (c->dv / (16 * nr)) <= c->num_sms;
+        rp.tile = std::min(longest, few ? kRecurMaxTail : kRecurTile);
+        const int ps = prof_begin(c, KVM_K_GDN, s);
+        launch_gdn_recur(rp, nr, s);
+        prof_end(c, ps, s);
+        LAUNCH_CHECK(c);
+        if (conv_inside) c->conv_par[g] ^= 1;
+        return KVM_OK;
+    }
+    thread_local static GdnParams p;
+    std::memset(&p, 0, sizeof p);
+    p.n_chars = c->B;
+    p.H = c->H; p.dk = c->dk; p.dv = c->dv;
+    // d_v rows of a head's state per scan block: split the rows (down to 32)
+    // until the (character, head, slice) blocks cover the SMs
+    {
+        int slices = 1;
+        while (c->dv / (2 * slices) >= 32 && c->dv % (2 * slices * 32) == 0 &&
+               (int64_t)active * c->H * slices < c->num_sms)
+            slices *= 2;
+        p.dv_slice = c->dv / slices;
+    }
+    p.q = static_cast<const __nv_bfloat16*>(q);
+    p.k = static_cast<const __nv_bfloat16*>(k);
+    p.v = static_cast<const __nv_bfloat16*>(v);
     p.alpha = alpha;
     p.beta = beta;
     p.out = static_cast<__nv_bfloat16*>(out);

@@ -260,6 +260,27 @@ struct ConvParams {
 };
 void launch_gdn_conv(const ConvParams& p, cudaStream_t s);
 
+// Token-by-token form of a delta-rule layer for short tails, with the short
+// convolution (w non-null) in the same launch.
+constexpr int kRecurMaxTail = 48;             // most tokens staged at once
+struct RecurParams {
+    int32_t n_chars, H, dk, dv, channels;     // channels: of the conv state
+    int32_t tile;                             // tokens staged at a time
+    int32_t tail_cu[kMaxChars + 1];
+    const __nv_bfloat16* q;                   // [sum M][H][d_k] (pre-convolution with w)
+    const __nv_bfloat16* k;
+    const __nv_bfloat16* v;                   // [sum M][H][d_v]
+    const float* alpha;                       // [sum M][H]
+    const float* beta;
+    __nv_bfloat16* out;                       // [sum M][H][d_v]
+    float* S;                                 // this layer's state [n_chars][H][d_v][d_k]
+    const float* w;                           // [channels][4], or null: no convolution
+    const __nv_bfloat16* state_in;            // [n_chars][3][channels], as in ConvParams
+    __nv_bfloat16* state_out;
+};
+// nr: rows of S per eight lanes (1, 2 or 4); 16 nr divides d_v.
+void launch_gdn_recur(const RecurParams& p, int nr, cudaStream_t s);
+
 // Bytes of one (chunk, head) record of the delta-rule workspace.
 int64_t gdn_record_bytes(int dk, int dv);
 void launch_gdn_chunk_prep(const GdnParams& p, cudaStream_t s);   // state-independent chunk products
