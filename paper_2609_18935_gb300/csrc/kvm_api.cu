@@ -348,13 +348,17 @@ kvm_status plan_spans(const kvm_ctx* c, const int32_t* span_cu, const int32_t* s
 // per-block cost target, found by bisection so that exactly G blocks cover
 // the units with the least maximum cost.  Tiles shared by several blocks are
 // merged once, from the first block that starts inside them (split_cb).
+// With `deal`, and more than a wave and a half of query tiles, the tiles up to
+// the last half to one and a half waves are dealt whole, one per block and
+// wave (see tail_attn_tc.cu), and only the rest is cut, each block's share
+// starting from the cost of what it was dealt.
 struct AttnPlan {
-    int n_tiles = 0, n_ctas = 0;
+    int n_tiles = 0, n_ctas = 0, waves = 0;
     std::vector<int> n_qtiles, tile_off;             // per character
     std::vector<int32_t> cta_tile, cta_k, split_cb;  // [n_ctas + 1], [n_ctas + 1], [number of split tiles]
 };
 
-void plan_attention(int B, const int* L_prev, const int* M, int Hkv, int tpt, int grid_cap, AttnPlan& pl) {
+void plan_attention(int B, const int* L_prev, const int* M, int Hkv, int tpt, int grid_cap, bool deal, AttnPlan& pl) {
     pl.n_qtiles.assign(B, 0);
     pl.tile_off.assign(B, 0);
     std::vector<int> nk_of;
@@ -377,28 +381,48 @@ void plan_attention(int B, const int* L_prev, const int* M, int Hkv, int tpt, in
     pl.n_ctas = G;
     pl.cta_tile.assign(G + 1, 0);
     pl.cta_k.assign(G + 1, 0);
+    pl.waves = 0;
+    std::vector<double> load(G, 0.0);                         // cost of each block's dealt tiles
+    if (deal && G == grid_cap) {
+        // another wave while no block passes its even share of all the work
+        // (the ranges level the rest): tiles of very uneven length are cut
+        const double share = ((double)units + kSegmentCost * tiles) / G;
+        for (std::vector<double> next = load; (pl.waves + 1) * G + G / 2 <= tiles; ++pl.waves) {
+            double most = 0.0;
+            for (int cc = 0; cc < G; ++cc) {
+                next[cc] += kSegmentCost + nk_of[pl.waves * G + ((pl.waves & 1) ? G - 1 - cc : cc)];
+                most = std::max(most, next[cc]);
+            }
+            if (most > share) break;
+            load = next;
+        }
+    }
+    const int first = pl.waves * G;                           // first tile that is not dealt
+    auto start_cost = [&](int block) { return (block < G ? load[block] : 0.0) + kSegmentCost; };
     // blocks needed to cover everything with ranges of cost <= target; the
     // cut points go to cta_tile / cta_k when `emit`
     auto cover = [&](double target, bool emit) -> int {
         int blocks = 1;
-        double cost = kSegmentCost;
-        for (int t = 0; t < (int)nk_of.size(); ++t) {
+        double cost = start_cost(0);
+        if (emit) { pl.cta_tile[0] = first; pl.cta_k[0] = 0; }
+        for (int t = first; t < (int)nk_of.size(); ++t) {
             int k = 0;
-            if (t > 0) cost += kSegmentCost;                  // entering a new query tile
+            if (t > first) cost += kSegmentCost;              // entering a new query tile
             while (k < nk_of[t]) {
                 const double room = target - cost;
                 const int take = room >= nk_of[t] - k ? nk_of[t] - k : std::max(0, (int)room);
                 k += take;
                 cost += take;
                 if (k < nk_of[t] && (take == 0 || cost >= target)) {
-                    if (take == 0 && cost == kSegmentCost) {      // a block must take at least a unit
+                    if (blocks > G) return blocks;                // more than there are
+                    if (take == 0 && cost == start_cost(blocks - 1)) {   // a block must take at least a unit
                         ++k;
                         cost += 1;
                         if (k >= nk_of[t]) break;
                     }
                     if (emit && blocks <= G) { pl.cta_tile[blocks] = t; pl.cta_k[blocks] = k; }
+                    cost = start_cost(blocks);
                     ++blocks;
-                    cost = kSegmentCost;
                 }
             }
         }
@@ -799,7 +823,7 @@ extern "C" kvm_status kvm_plan_attention(int32_t n_chars, const int32_t* live, c
         if (L[b] < 0) return fail(KVM_E_INVAL, "negative live length at character %d", b);
     }
     AttnPlan pl;
-    plan_attention(n_chars, L.data(), M.data(), n_kv_heads, kAttnRows / g, max_blocks, pl);
+    plan_attention(n_chars, L.data(), M.data(), n_kv_heads, kAttnRows / g, max_blocks, false, pl);
     *n_blocks = pl.n_ctas;
     *n_tiles = pl.n_tiles;
     std::copy(pl.cta_tile.begin(), pl.cta_tile.end(), block_tile);
@@ -1068,18 +1092,16 @@ kvm_status do_attention(kvm_ctx* c, int layer, const int32_t* tail_cu, const voi
         ch.p = c->cursor[b];
     }
     AttnPlan pl;
-    plan_attention(c->B, c->live.data(), Ms.data(), c->Hkv, p.tok_per_tile, attention_grid_cap(c->num_sms, c->D), pl);
+    plan_attention(c->B, c->live.data(), Ms.data(), c->Hkv, p.tok_per_tile, attention_grid_cap(c->num_sms, c->D), true, pl);
     for (int b = 0; b < c->B; ++b) {
         p.ch[b].n_qtiles = pl.n_qtiles[b];
         p.ch[b].tile_off = pl.tile_off[b];
     }
     p.n_tiles = pl.n_tiles;
     p.n_ctas = pl.n_ctas;
+    p.waves = pl.waves;
     std::copy(pl.cta_tile.begin(), pl.cta_tile.end(), p.cta_tile);
     std::copy(pl.cta_k.begin(), pl.cta_k.end(), p.cta_k);
-    p.n_split_tiles = (int)pl.split_cb.size();
-    std::copy(pl.split_cb.begin(), pl.split_cb.end(), p.split_cb);
-    const bool split_tiles = p.n_split_tiles > 0;
 
     int ps = prof_begin(c, KVM_K_ROPE_APPEND, s);
     launch_rope_append(p, total, s);
@@ -1089,9 +1111,31 @@ kvm_status do_attention(kvm_ctx* c, int layer, const int32_t* tail_cu, const voi
     launch_tail_attention(p, s);
     prof_end(c, ps, s);
     LAUNCH_CHECK(c);
-    if (split_tiles) {
+    if (!pl.split_cb.empty()) {
+        thread_local static CombineParams cp;
+        cp.Hq = c->Hq; cp.D = c->D; cp.g = c->g;
+        cp.n_split_tiles = (int)pl.split_cb.size();
+        cp.part_o = c->part_o;
+        cp.part_ml = c->part_ml;
+        cp.out = p.out;
+        int b = 0;                                   // tiles come in order
+        for (int x = 0; x < cp.n_split_tiles; ++x) {
+            // blocks c0 .. c1 hold the tile: c0 starts before or at it, the others inside
+            const int cb = pl.split_cb[x], t = pl.cta_tile[cb], c0 = cb - 1;
+            int c1 = cb;
+            while (c1 + 1 < pl.n_ctas && pl.cta_tile[c1 + 1] == t && pl.cta_k[c1 + 1] > 0) ++c1;
+            while (pl.n_qtiles[b] == 0 || t >= pl.tile_off[b] + c->Hkv * pl.n_qtiles[b]) ++b;
+            const int local = t - pl.tile_off[b], tok = local % pl.n_qtiles[b] * p.tok_per_tile;
+            SplitTile& st = cp.tile[x];
+            st.block0 = (int16_t)c0;
+            st.n_parts = (int16_t)(c1 - c0 + 1);
+            st.slot0 = pl.cta_tile[c0] == t ? 2 * c0 : 2 * c0 + 1;
+            st.token0 = tail_cu[b] + tok;
+            st.rows = (int16_t)(std::min(p.tok_per_tile, Ms[b] - tok) * c->g);
+            st.head0 = (int16_t)(local / pl.n_qtiles[b] * c->g);
+        }
         ps = prof_begin(c, KVM_K_ATTN_COMBINE, s);
-        launch_attn_combine(p, s);
+        launch_attn_combine(cp, s);
         prof_end(c, ps, s);
         LAUNCH_CHECK(c);
     }

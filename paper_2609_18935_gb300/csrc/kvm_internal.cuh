@@ -118,8 +118,10 @@ struct AttnChar {
 };
 
 // The attention's work is the list of (query tile, 64-key tile) units, query
-// tiles in order and each tile's key tiles in order; persistent block c
-// processes units [start_c, start_{c+1}), given as (query tile, key tile).
+// tiles in order and each tile's key tiles in order.  The first waves * n_ctas
+// query tiles are dealt whole, one per block and wave (odd waves in reverse
+// block order); of the rest, persistent block c processes units
+// [start_c, start_{c+1}), given as (query tile, key tile).
 constexpr int kMaxAttnCtas = 320;
 
 struct AttnParams {
@@ -131,6 +133,7 @@ struct AttnParams {
     int32_t Hq, Hkv, D, R, g;
     int32_t n_tiles;      // query tiles over all characters and KV heads
     int32_t n_ctas;       // persistent attention blocks
+    int32_t waves;        // whole query tiles dealt to every block first
     int32_t tok_per_tile; // tail tokens per 128-row query tile (128 / g)
     float scale_log2;     // log2(e) / sqrt(D)
     int64_t slab_rows;    // rows per (layer, head) slab
@@ -150,9 +153,25 @@ struct AttnParams {
     double inv_freq[kMaxRotaryHalf];
     int32_t cta_tile[kMaxAttnCtas + 1];
     int32_t cta_k[kMaxAttnCtas + 1];
-    int32_t n_split_tiles;                   // query tiles shared by several blocks
-    int32_t split_cb[kMaxAttnCtas];          // per such tile: the first block that starts inside it
     AttnChar ch[kMaxChars];
+};
+
+// A query tile shared by several attention blocks: its parts are in slot0 and
+// in slots 2 (block0 + q), 0 < q < n_parts; its real rows (token-major, then
+// the group's heads) are output rows of tokens token0 .. and heads head0 ..
+struct SplitTile {
+    int32_t slot0;
+    int32_t token0;
+    int16_t block0, n_parts;
+    int16_t rows, head0;
+};
+struct CombineParams {
+    int32_t Hq, D, g;
+    int32_t n_split_tiles;
+    const float* part_o;          // as in AttnParams
+    const float* part_ml;
+    __nv_bfloat16* out;           // [sum M][Hq][D]
+    SplitTile tile[kMaxAttnCtas];
 };
 
 void launch_rope_append(const AttnParams& p, int total_tokens, cudaStream_t s);
@@ -172,7 +191,7 @@ struct RerotateParams {
 };
 void launch_rerotate(const RerotateParams& p, cudaStream_t s);
 void launch_tail_attention(const AttnParams& p, cudaStream_t s);
-void launch_attn_combine(const AttnParams& p, cudaStream_t s);
+void launch_attn_combine(const CombineParams& p, cudaStream_t s);
 int attention_ctas_per_sm(int head_dim);
 constexpr int kAttnRows = 128;   // query rows per attention tile
 

@@ -169,46 +169,30 @@ __global__ void __launch_bounds__(128) rope_append_kernel(const __grid_constant_
     if (threadIdx.x == 0) p.pos[slot] = (int32_t)pos;
 }
 
-// grid (n_split_tiles, kRows * D / 4 / 256): the x-th query tile that several
-// attention blocks share.  Block cb = split_cb[x] is the first to start
-// inside the tile, so its partials are in the slots of blocks c0 = cb - 1 ..
-// c1 (the last block that starts inside the tile): c0's last segment (slot
-// 2 c0 + 1, or 2 c0 when the tile is also c0's first segment) and the first
-// segments 2 c of the others.  A thread owns four columns of one row (rows
-// fastest across threads, as in the partial layout) and merges the partials
-// online, two at a time, each batch's (max, sum) pairs and O pieces loaded
-// together.
+// Slot of part q of a shared tile: the first block's last (or only) range
+// segment, then the first range segments of the blocks after it.
+__device__ __forceinline__ int part_slot(const SplitTile& s, int q) { return q == 0 ? s.slot0 : 2 * (s.block0 + q); }
+
+// grid (n_split_tiles, kRows * D / 4 / 256): a thread owns four columns of one
+// row (rows fastest across threads, as in the partial layout) and merges the
+// partials online, two at a time, each batch's (max, sum) pairs and O pieces
+// loaded together.
 // At most 36 registers a thread keep seven blocks on an SM, so that the
 // grid of a round with up to 33 shared tiles (x 32 blocks at head_dim 256)
 // runs in one wave.
-__global__ void __launch_bounds__(256, 7) attn_combine_piece_kernel(const __grid_constant__ AttnParams p) {
+__global__ void __launch_bounds__(256, 7) attn_combine_piece_kernel(const __grid_constant__ CombineParams p) {
     grid_dependency_wait();
     grid_dependents_launch();
-    const int cb = p.split_cb[blockIdx.x];
-    const int t = p.cta_tile[cb];
-    const int c0 = cb - 1;
-    int c1 = cb;
-    while (c1 + 1 < p.n_ctas && p.cta_tile[c1 + 1] == t && p.cta_k[c1 + 1] > 0) ++c1;
-    const int slot0 = (p.cta_tile[c0] == t) ? 2 * c0 : 2 * c0 + 1;
-    const int n_parts = c1 - c0 + 1;
-
-    int lo = 0, hi = p.n_chars - 1;                                // last b with tile_off <= t
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (p.ch[mid].tile_off <= t) lo = mid; else hi = mid - 1;
-    }
-    const AttnChar& c = p.ch[lo];
-    const int local = t - c.tile_off;
-    const int kvh = local / c.n_qtiles, qt = local % c.n_qtiles;
+    const SplitTile st = p.tile[blockIdx.x];
+    const int n_parts = st.n_parts;
     const int D = p.D;
     const int item = blockIdx.y * blockDim.x + threadIdx.x;        // (4-column piece, row): rows fastest
     const int r = item % kRows;
     const int piece = item / kRows;
     if (piece >= D / 4) return;
     const int cg = piece >> 3, q4 = piece & 7;
-    const int tok = qt * p.tok_per_tile + r / p.g;
-    if (tok >= c.M) return;
-    __nv_bfloat16* o = p.out + ((int64_t)(c.tail_off + tok) * p.Hq + kvh * p.g + (r % p.g)) * D + cg * 32 + q4 * 4;
+    if (r >= st.rows) return;
+    __nv_bfloat16* o = p.out + ((int64_t)(st.token0 + r / p.g) * p.Hq + st.head0 + r % p.g) * D + cg * 32 + q4 * 4;
     // this thread's piece of slot s: po + s * D * kRows floats; its (max, sum): pm + s * 2 kRows
     const float* po = p.part_o + ((cg * 8 + q4) * kRows + r) * 4;
     const float* pm = p.part_ml + r * 2;
@@ -222,7 +206,7 @@ __global__ void __launch_bounds__(256, 7) attn_combine_piece_kernel(const __grid
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             if (q0 + u < n_parts) {
-                const int slot = (q0 + u == 0) ? slot0 : 2 * (c0 + q0 + u);
+                const int slot = part_slot(st, q0 + u);
                 ml[u] = *reinterpret_cast<const float2*>(pm + slot * (2 * kRows));
                 x[u] = *reinterpret_cast<const float4*>(po + slot * sstride);
             } else {
@@ -250,43 +234,23 @@ __global__ void __launch_bounds__(256, 7) attn_combine_piece_kernel(const __grid
     *reinterpret_cast<uint2*>(o) = make_uint2(f2_to_bf2(acc.x * inv, acc.y * inv), f2_to_bf2(acc.z * inv, acc.w * inv));
 }
 
-// grid (n_split_tiles, kRows * D / 32 / kCombineThreads): the x-th query
-// tile that several attention blocks share.  Block cb = split_cb[x] is the
-// first to start inside the tile, so its partials are in the slots of blocks
-// c0 = cb - 1 .. c1 (the last block that starts inside the tile): c0's last
-// segment (slot 2 c0 + 1, or 2 c0 when the tile is also c0's first segment)
-// and the first segments 2 c of the others.  A thread owns one 32-column
-// group of one row (rows fastest across threads, as in the partial layout)
-// and merges the partials online, two at a time: both (max, sum) pairs
-// first, then each part's eight 4-column pieces.
+// grid (n_split_tiles, kRows * D / 32 / kCombineThreads): a thread owns one
+// 32-column group of one row (rows fastest) and merges the partials online,
+// two at a time: both (max, sum) pairs first, then each part's eight 4-column
+// pieces.
 constexpr int kCombineThreads = 128;
-__global__ void __launch_bounds__(kCombineThreads) attn_combine_group_kernel(const __grid_constant__ AttnParams p) {
+__global__ void __launch_bounds__(kCombineThreads) attn_combine_group_kernel(const __grid_constant__ CombineParams p) {
     grid_dependency_wait();
     grid_dependents_launch();
-    const int cb = p.split_cb[blockIdx.x];
-    const int t = p.cta_tile[cb];
-    const int c0 = cb - 1;
-    int c1 = cb;
-    while (c1 + 1 < p.n_ctas && p.cta_tile[c1 + 1] == t && p.cta_k[c1 + 1] > 0) ++c1;
-    const int slot0 = (p.cta_tile[c0] == t) ? 2 * c0 : 2 * c0 + 1;
-    const int n_parts = c1 - c0 + 1;
-
-    int lo = 0, hi = p.n_chars - 1;                                // last b with tile_off <= t
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (p.ch[mid].tile_off <= t) lo = mid; else hi = mid - 1;
-    }
-    const AttnChar& c = p.ch[lo];
-    const int local = t - c.tile_off;
-    const int kvh = local / c.n_qtiles, qt = local % c.n_qtiles;
+    const SplitTile st = p.tile[blockIdx.x];
+    const int n_parts = st.n_parts;
     const int D = p.D;
     const int item = blockIdx.y * blockDim.x + threadIdx.x;        // (column group, row): rows fastest
     const int r = item % kRows;
     const int cg = item / kRows;
     if (cg >= D / 32) return;
-    const int tok = qt * p.tok_per_tile + r / p.g;
-    if (tok >= c.M) return;
-    __nv_bfloat16* o = p.out + ((int64_t)(c.tail_off + tok) * p.Hq + kvh * p.g + (r % p.g)) * D + cg * 32;
+    if (r >= st.rows) return;
+    __nv_bfloat16* o = p.out + ((int64_t)(st.token0 + r / p.g) * p.Hq + st.head0 + r % p.g) * D + cg * 32;
     // piece q4 of slot s: po + s * D * kRows + q4 * 4 kRows floats; (max, sum): pm + s * 2 kRows
     const float* po = p.part_o + (cg * 8 * kRows + r) * 4;
     const float* pm = p.part_ml + r * 2;
@@ -301,8 +265,8 @@ __global__ void __launch_bounds__(kCombineThreads) attn_combine_group_kernel(con
         int slot[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
-            slot[u] = (q0 + u == 0) ? slot0 : 2 * (c0 + q0 + u);
-            ml[u] = (q0 + u < n_parts) ? *reinterpret_cast<const float2*>(pm + slot[u] * (2 * kRows))
+            slot[u] = part_slot(st, q0 + u);
+            ml[u] = q0 + u < n_parts ? *reinterpret_cast<const float2*>(pm + slot[u] * (2 * kRows))
                                        : make_float2(-INFINITY, 0.f);
         }
         float bm = -INFINITY;
@@ -337,6 +301,67 @@ __global__ void __launch_bounds__(kCombineThreads) attn_combine_group_kernel(con
                                                     f2_to_bf2(acc[2 * e].z * inv, acc[2 * e].w * inv),
                                                     f2_to_bf2(acc[2 * e + 1].x * inv, acc[2 * e + 1].y * inv),
                                                     f2_to_bf2(acc[2 * e + 1].z * inv, acc[2 * e + 1].w * inv));
+}
+
+// Few rows, many parts (decode steps): a query tile of a single token has g
+// rows, and one character's tiles are split over tens of blocks.  A warp of
+// the block takes every 16th part for 32 (row, 4-column piece) items, rows
+// fastest; the 16 results meet in shared memory.  grid (n_split_tiles,
+// ceil(largest tile's rows * D / 4 / 32)).
+constexpr int kPartLanes = 16;
+__global__ void __launch_bounds__(32 * kPartLanes) attn_combine_parts_kernel(const __grid_constant__ CombineParams p) {
+    grid_dependency_wait();
+    grid_dependents_launch();
+    __shared__ float4 acc_s[kPartLanes][32];
+    __shared__ float2 md_s[kPartLanes][32];
+    const SplitTile st = p.tile[blockIdx.x];
+    const int D = p.D, rows = st.rows;
+    const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+    const int item = blockIdx.y * 32 + lane;
+    if ((int)blockIdx.y * 32 >= rows * (D / 4)) return;                         // uniform per block
+    const bool act = item < rows * (D / 4);
+    const int r = act ? item % rows : 0, piece = act ? item / rows : 0;
+    const float* po = p.part_o + ((int64_t)piece * kRows + r) * 4;
+    const float* pm = p.part_ml + r * 2;
+    const int sstride = D * kRows;
+    float mx = -INFINITY, den = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto merge = [&](const float2& ml, const float4& x) {
+        if (ml.x == -INFINITY) return;
+        const float nmx = fmaxf(mx, ml.x);
+        const float sc = (mx == -INFINITY) ? 0.f : exp2f(mx - nmx), w = exp2f(ml.x - nmx);
+        den = den * sc + w * ml.y;
+        acc.x = acc.x * sc + w * x.x; acc.y = acc.y * sc + w * x.y;
+        acc.z = acc.z * sc + w * x.z; acc.w = acc.w * sc + w * x.w;
+        mx = nmx;
+    };
+#pragma unroll 2
+    for (int q = part; q < st.n_parts; q += kPartLanes) {
+        const int slot = part_slot(st, q);
+        const float2 ml = *reinterpret_cast<const float2*>(pm + slot * (2 * kRows));
+        const float4 x = *reinterpret_cast<const float4*>(po + (int64_t)slot * sstride);
+        merge(ml, x);
+    }
+    acc_s[part][lane] = acc;
+    md_s[part][lane] = make_float2(mx, den);
+    __syncthreads();
+    if (part > 0 || !act) return;
+    float top = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < kPartLanes; ++q) top = fmaxf(top, md_s[q][lane].x);
+    den = 0.f;
+    acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < kPartLanes; ++q) {
+        const float2 md = md_s[q][lane];
+        const float4 x = acc_s[q][lane];
+        const float w = md.x == -INFINITY ? 0.f : exp2f(md.x - top);
+        den += w * md.y;
+        acc.x += w * x.x; acc.y += w * x.y; acc.z += w * x.z; acc.w += w * x.w;
+    }
+    const float inv = den > 0.f ? 1.f / den : 0.f;
+    __nv_bfloat16* o = p.out + ((int64_t)(st.token0 + r / p.g) * p.Hq + st.head0 + r % p.g) * D + piece * 4;
+    *reinterpret_cast<uint2*>(o) = make_uint2(f2_to_bf2(acc.x * inv, acc.y * inv), f2_to_bf2(acc.z * inv, acc.w * inv));
 }
 
 // One block per entry; a thread rotates 2-element pairs (d, d + R/2) of one
@@ -383,16 +408,28 @@ void launch_rope_append(const AttnParams& p, int total_tokens, cudaStream_t s) {
     launch_pdl(rope_append_kernel, dim3(total_tokens), dim3(128), 0, s, p);
 }
 
-void launch_attn_combine(const AttnParams& p, cudaStream_t s) {
+void launch_attn_combine(const CombineParams& p, cudaStream_t s) {
     if (p.n_split_tiles <= 0) return;
     // one 4-column piece a thread while that grid is one wave (seven blocks
     // an SM), else a 32-column group a thread: at npc (32 shared tiles) the
-    // piece form took 11.0 against 12.4 us, at long (128) 16.3 against 13.1
+    // piece form took 11.0 against 12.4 us (6.9 now that the host hands each
+    // shared tile over as one record), at long (128) 16.3 against 13.1 (11.3)
     static int sms_of[64] = {};                      // per device
     int dev = 0;
     cudaGetDevice(&dev);
     int& sms = sms_of[dev & 63];
     if (!sms) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // few real rows in a tile (decode steps): parts side by side, while that
+    // grid is two waves (four blocks an SM).  One character's step at 8K (two
+    // tiles, 32 parts each) 4.0 us against 13 in the piece form; with all 128
+    // rows real and two parts (a 64-token tail at head_dim 64) 3.6 against 2.8
+    int rows = 0;
+    for (int x = 0; x < p.n_split_tiles; ++x) rows = max(rows, (int)p.tile[x].rows);
+    const int part_blocks = (rows * (p.D / 4) + 31) / 32;
+    if (rows <= 32 && (int64_t)p.n_split_tiles * part_blocks <= 8 * (int64_t)sms) {
+        launch_pdl(attn_combine_parts_kernel, dim3(p.n_split_tiles, part_blocks), dim3(32 * kPartLanes), 0, s, p);
+        return;
+    }
     const int piece_blocks = (kRows * (p.D / 4) + 255) / 256;
     if ((int64_t)p.n_split_tiles * piece_blocks <= 7 * (int64_t)sms)
         launch_pdl(attn_combine_piece_kernel, dim3(p.n_split_tiles, piece_blocks), dim3(256), 0, s, p);

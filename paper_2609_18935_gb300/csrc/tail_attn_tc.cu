@@ -3,13 +3,21 @@
 //
 // Query tiles have 128 rows = (tail token, query head of one GQA group) pairs,
 // token-major, so each K/V tile serves all g heads of the group.  The work is
-// the list of (query tile, 64-key tile) units; it is cut into contiguous
-// ranges, one per persistent block (stream-K), balanced by a cost model that
+// the list of (query tile, 64-key tile) units.  While there is more than a
+// wave and a half of query tiles, whole tiles are dealt to the persistent
+// blocks, one a wave: neighbouring tiles of a character's KV head then run on
+// neighbouring blocks at the same time, from its first key on, and share its
+// K/V through L2.  With contiguous ranges alone each block streamed the keys
+// again for every tile of its range: 32 characters' 544 MB of K/V cost 9.2 GB of
+// DRAM reads (2.9 now) and the layer 1340 us (1015 now), a 16896-token prefill
+// 1790 us (1660 now).
+// The rest is cut into contiguous ranges, one per block (stream-K), balanced by a
+// cost model that
 // charges each unit 1 and each segment a block starts 8 more (the host
 // planner bisects for the smallest per-block cost).  A block's range covers whole
 // query tiles, whose outputs it normalises and stores directly, and at most
 // one partial tile at each end, whose unnormalised accumulator goes to a
-// workspace slot (2c for block c's first segment, 2c + 1 for its last) for
+// workspace slot (2c for block c's first range segment, 2c + 1 for its last) for
 // attn_combine.
 //
 // Roles of a block (384 threads):
@@ -115,7 +123,9 @@ __device__ __forceinline__ Tile decode_tile(const AttnParams& p, int t) {
     return r;
 }
 
-template <int D>
+// DEAL: p.waves > 0 (a kernel of its own: the segment lookup with waves cost
+// 1 % of the time where there are none)
+template <int D, bool DEAL>
 __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __grid_constant__ AttnParams p) {
     using C = Cfg<D>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -136,9 +146,18 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = blockIdx.x;
     const int g = p.g;
+    // the block's segments: one whole query tile of each dealt wave (odd waves
+    // in reverse block order), then those of its contiguous range
     const int t_begin = p.cta_tile[cta], k_begin = p.cta_k[cta];
     const int t_end = p.cta_tile[cta + 1], k_end = p.cta_k[cta + 1];
-    auto more = [&](int t, int k) { return t < t_end || (t == t_end && k < k_end); };
+    const int waves = DEAL ? p.waves : 0;
+    const int n_seg = waves + ((t_begin == t_end && k_begin == k_end) ? 0 : t_end - t_begin + (k_end > 0 ? 1 : 0));
+    auto tile_of = [&](int seg) {
+        return seg < waves ? seg * p.n_ctas + ((seg & 1) ? p.n_ctas - 1 - cta : cta) : t_begin + (seg - waves);
+    };
+    // first key tile of a segment, and one past its last (nk: of the query tile)
+    auto key_begin = [&](int seg) { return seg == waves ? k_begin : 0; };
+    auto key_end = [&](int seg, int nk) { return (seg >= waves && t_begin + (seg - waves) == t_end) ? k_end : nk; };
     // A barrier wait of a whole issuer warp: lane 0 polls, the warp takes its result.
     auto warp_wait = [&](uint32_t b, uint32_t parity, int tag) -> bool {
         int r = 1;
@@ -196,10 +215,10 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
             prefetch_tmap(map);
             bool ok = true, waited = false;
             int j = 0;
-            for (int t = t_begin, k = k_begin; ok && more(t, k); ++t, k = 0) {
-                const Tile T = decode_tile(p, t);
+            for (int seg = 0; ok && seg < n_seg; ++seg) {
+                const Tile T = decode_tile(p, tile_of(seg));
                 const AttnChar& ch = p.ch[T.b];
-                const int k1 = (t == t_end) ? k_end : T.nk;
+                const int k = key_begin(seg), k1 = key_end(seg, T.nk);
                 const int key_row0 = (p.attn_layer * p.Hkv + T.kvh) * (int)p.slab_rows + ch.cap_off;
                 for (int kt = k; kt < k1; ++kt, ++j) {
                     if (!waited && (kt + 1) * BN > ch.L_prev) {    // the tile reaches the tail
@@ -226,10 +245,10 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
         const uint32_t id_qk = idesc_bf16_f32(BM, BN, false);
         const uint64_t k_desc0 = smem_desc_sw128(sK, 16, 1024);   // + (byte offset >> 4) per operand
         bool ok = true;
-        int j = 0, seg = 0;
-        for (int t = t_begin, k = k_begin; ok && more(t, k); ++t, k = 0, ++seg) {
-            const Tile T = decode_tile(p, t);
-            const int n = ((t == t_end) ? k_end : T.nk) - k;
+        int j = 0;
+        for (int seg = 0; ok && seg < n_seg; ++seg) {
+            const Tile T = decode_tile(p, tile_of(seg));
+            const int n = key_end(seg, T.nk) - key_begin(seg);
             ok = warp_wait(bar(Q_FULL), seg & 1, 0x21 + 256 * seg);
             for (int i = 0; i < n && ok; ++i, ++j) {
                 const int sb = j & 1, st = j % STAGES;
@@ -262,10 +281,10 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
         const uint64_t p_desc0 = smem_desc_sw128(sP, 16, 1024);
         const uint64_t v_desc0 = smem_desc_sw128(sV, BN * 128, 1024);
         bool ok = true;
-        int j = 0, seg = 0;
-        for (int t = t_begin, k = k_begin; ok && more(t, k); ++t, k = 0, ++seg) {
-            const Tile T = decode_tile(p, t);
-            const int n = ((t == t_end) ? k_end : T.nk) - k;
+        int j = 0;
+        for (int seg = 0; ok && seg < n_seg; ++seg) {
+            const Tile T = decode_tile(p, tile_of(seg));
+            const int n = key_end(seg, T.nk) - key_begin(seg);
             for (int i = 0; i < n && ok; ++i, ++j) {
                 const int pb = j & 1, st = j % STAGES;
                 ok = warp_wait(bar(P_FULL + pb), (j >> 1) & 1, 0x24 + 256 * j);
@@ -349,15 +368,15 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
             tc_fence_before();
             mbar_arrive(bar(Q_FULL));
         };
-        if (more(t_begin, k_begin)) stage_q(t_begin);
-        int j = 0, seg = 0;
-        for (int t = t_begin, k = k_begin; more(t, k); ++t, k = 0, ++seg) {
-            const Tile T = decode_tile(p, t);
+        if (n_seg > 0) stage_q(tile_of(0));
+        int j = 0;
+        for (int seg = 0; seg < n_seg; ++seg) {
+            const Tile T = decode_tile(p, tile_of(seg));
             const AttnChar& ch = p.ch[T.b];
-            const int k1 = (t == t_end) ? k_end : T.nk;
+            const int k = key_begin(seg), k1 = key_end(seg, T.nk);
             const int n = k1 - k;
             const bool full = (k == 0 && k1 == T.nk);
-            const bool has_next = more(t + 1, 0);
+            const bool has_next = seg + 1 < n_seg;
             const int tok = T.tok0 + r / g;
             const bool row_valid = tok < ch.M;
             const int lim = ch.L_prev + min(tok, ch.M - 1) + 1;    // keys [0, lim) are visible
@@ -373,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
                 tc_fence_before();
                 mbar_arrive(bar(S_EMPTY + sb));
                 // the segment's last S has landed, so no MMA reads Q any more
-                if (i + 1 == n && has_next) stage_q(t + 1);
+                if (i + 1 == n && has_next) stage_q(tile_of(seg + 1));
                 const int key0 = (k + i) * BN + 32 * half;
                 float s[32];
 #pragma unroll
@@ -484,20 +503,20 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
                     }
                 }
             } else {
-                const int64_t prow = (int64_t)(2 * cta + (seg == 0 ? 0 : 1)) * BM + r;
-                if (half == 0 && store) {
+                const int64_t prow = (int64_t)(2 * cta + (seg == waves ? 0 : 1)) * BM + r;
+                if (half == 0 && store && row_valid) {       // only real rows are merged
                     p.part_ml[prow * 2 + 0] = mr;
                     p.part_ml[prow * 2 + 1] = lt;
                 }
                 // partial layout [slot][D / 32][8][row][4]: each 16-byte store
                 // of a warp lands in 512 contiguous bytes
-                const int64_t slot = 2 * cta + (seg == 0 ? 0 : 1);
+                const int64_t slot = 2 * cta + (seg == waves ? 0 : 1);
 #pragma unroll 1
                 for (int c0 = half * C::HALF; c0 < (half + 1) * C::HALF; c0 += 32) {
                     uint32_t v[32];
                     tmem_ld32(tmem + lane_off + C::TMEM_O + c0, v);
                     tmem_ld_wait();
-                    if (store) {
+                    if (store && row_valid) {
                         uint4* dst = reinterpret_cast<uint4*>(p.part_o + (slot * (D / 32) + c0 / 32) * 8 * BM * 4) + r;
 #pragma unroll
                         for (int e = 0; e < 8; ++e)
@@ -526,17 +545,17 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
     }
 }
 
-template <int D>
+template <int D, bool DEAL>
 void launch_tc(const AttnParams& p, cudaStream_t s) {
     using C = Cfg<D>;
     static unsigned long long configured = 0;   // one bit per device
     int dev = 0;
     cudaGetDevice(&dev);
     if (!(configured >> (dev & 63) & 1ull)) {
-        cudaFuncSetAttribute(tail_attention_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        cudaFuncSetAttribute(tail_attention_tc_kernel<D, DEAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
         configured |= 1ull << (dev & 63);
     }
-    launch_pdl(tail_attention_tc_kernel<D>, dim3(p.n_ctas), dim3(kThreads), C::SMEM, s, p);
+    launch_pdl(tail_attention_tc_kernel<D, DEAL>, dim3(p.n_ctas), dim3(kThreads), C::SMEM, s, p);
 }
 
 }  // namespace
@@ -544,9 +563,9 @@ void launch_tc(const AttnParams& p, cudaStream_t s) {
 void launch_tail_attention(const AttnParams& p, cudaStream_t s) {
     if (p.n_ctas <= 0) return;
     switch (p.D) {
-        case 64: launch_tc<64>(p, s); break;
-        case 128: launch_tc<128>(p, s); break;
-        case 256: launch_tc<256>(p, s); break;
+        case 64: p.waves > 0 ? launch_tc<64, true>(p, s) : launch_tc<64, false>(p, s); break;
+        case 128: p.waves > 0 ? launch_tc<128, true>(p, s) : launch_tc<128, false>(p, s); break;
+        case 256: p.waves > 0 ? launch_tc<256, true>(p, s) : launch_tc<256, false>(p, s); break;
         default: break;   // rejected on the host
     }
 }
