@@ -1580,12 +1580,15 @@ __device__ __forceinline__ void gdn_scan_packed_run(const GdnParams& p, const Fu
             }
         }
     };
+    // A fused launch's previous kernel may be the same layer's (a stack of one
+    // recurrent layer): its state is only complete after the wait.
+    if (fc.flags) grid_dependency_wait();
     float sreg[CW];
 #pragma unroll
     for (int j = 0; j < CW; ++j)                     // all loads before any use
         sreg[j] = (cols && row < DK && rc + j < dvs) ? Sg[(int64_t)(r0 + rc + j) * DK + row] : 0.f;
     if (cols && row < DK) write_s(row, sreg);
-    // The state slice comes from an earlier round (or kvm_set_state), which
+    // Launched after a prep kernel, the state slice comes from an earlier round (or kvm_set_state), which
     // completed before the prep kernel this launch follows had started, so
     // it is staged before waiting for that kernel; its records are not.
     grid_dependency_wait();
