@@ -103,8 +103,45 @@ __device__ __forceinline__ int find_char_by_chunk(const GdnParams& p, int chunk)
 // ============================================================================
 constexpr int kPrepThreads = 512;
 
-template <int DK>
+// Shared memory and tensor memory of a prep block.  PER_SM 2: 114 KB and 256
+// columns, so that two blocks share an SM and one's loads, solve and stores run
+// beside the other's products (each phase waits on the one before it, and a
+// block alone leaves the SM idle most of the time).  PER_SM 1 (grids of at most
+// a block an SM, and fused launches): U | A U staged in space of its own.
+template <int DK, int PER_SM>
 struct PrepCfg {
+    static constexpr int KQ = 128 * DK * 2;                  // [K;Q] bf16, K-major, 128 rows
+    static constexpr int V = C * DVMAX * 2;                  // V bf16, rows j (MN-major operand)
+    static constexpr int TILE128 = 128 * 64 * 2;             // 128 x 64 bf16 K-major tile
+    static constexpr int OFF_KQ = 0;
+    static constexpr int OFF_V = OFF_KQ + KQ;
+    static constexpr int OFF_XG = OFF_V + V;                 // [I; A] hi, lo, then X G hi, lo
+    static constexpr int OFF_X = OFF_XG + 2 * TILE128;       // T hi, lo (MN-major) and L, then X hi, lo
+    static constexpr int OFF_L = OFF_X + TILE128;            // L (strictly lower), fp32 [64][64]
+    static constexpr int OFF_G = OFF_X + 2 * TILE128;        // G, beta, log2 G: fp32 [64] each
+    static constexpr int OFF_BAR = OFF_G + 3 * C * 4;        // barrier, TMEM address, abort flag
+    static constexpr int OFF_END = OFF_BAR + 64;
+    static constexpr int U_PIECE = 128 * 64 * 4;             // 64 columns of U | A U
+    // no static shared memory: the dynamic base is 1024-aligned
+    static constexpr int SMEM = PER_SM == 2 ? OFF_END : OFF_END + 2 * U_PIECE;
+    // record staging: [W;Q'] hi | lo over XG, X; U | A U in two pieces of 64
+    // columns, with PER_SM 2 the first over [K;Q] (and V), the second over what
+    // [W;Q'] hi (at d_k 64: nothing any more) was staged in
+    static constexpr int OFF_STAGE_WQ = OFF_XG;
+    static constexpr int OFF_STAGE_U0 = PER_SM == 2 ? OFF_KQ : OFF_END;
+    static constexpr int OFF_STAGE_U1 = PER_SM == 2 ? (DK == 128 ? OFF_XG : OFF_X) : OFF_END + U_PIECE;
+    static_assert(OFF_XG % 1024 == 0 && OFF_V % 1024 == 0, "operand tiles on 1024-byte boundaries");
+    static_assert(2 * 128 * DK * 2 <= 4 * TILE128, "[W;Q'] staging");
+    static_assert(U_PIECE <= KQ + V && OFF_END % 16 == 0, "U | A U staging");
+    static_assert(PER_SM * (SMEM + 1024) <= 228 * 1024, "blocks an SM");
+    static constexpr uint32_t T_D = 0;                       // KK / QK, then X (64 cols)
+    static constexpr uint32_t T_WU = 0;                      // [W | U] (DK + dv cols), over X (consumed)
+    static constexpr uint32_t T_COLS = 256;
+};
+constexpr int LST = 64;          // fp32 row stride of L: the solve's threads read neighbouring columns
+
+template <int DK>
+struct PrepWide {
     static constexpr int KQ = 128 * DK * 2;                  // [K;Q] bf16, K-major, 128 rows
     static constexpr int V = C * DVP * 2;                    // V bf16, rows j (MN-major operand)
     static constexpr int TILE128 = 128 * 64 * 2;             // 128 x 64 bf16 K-major tile
@@ -154,7 +191,7 @@ __device__ __forceinline__ int au_idx(int row, int col) { return ((col >> 5) * 6
 
 template <int DK>
 struct Prep2Cfg {
-    using G = PrepCfg<DK>;
+    using G = PrepWide<DK>;
     static constexpr uint32_t WW_HALF = 64 * DK * 2;         // w W operand half [64 tokens][DK]
     static constexpr uint32_t WU_HALF = 64 * 128 * 2;        // w U operand half [64 tokens][dv <= 128]
     static constexpr uint32_t OFF_WW = G::OFF_XG;            // over the X G tiles (consumed)
@@ -248,12 +285,19 @@ __device__ __forceinline__ int fused_unit(const GdnParams& p, int u) {
 // The prep's work units u = u0, u0 + ustride, ... (standalone: one unit per
 // block, u = blockIdx.x over (chunk, head, part); fused: the units of
 // fused_unit, one part each).
-template <int DK>
+template <int DK, int PER_SM>
 __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& fc, int u0, int ustride) {
-    using G = PrepCfg<DK>;
+    using G = PrepCfg<DK, PER_SM>;
     using R = Rec<DK>;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    // a launch of its own has no static shared memory and no room to align up;
+    // a fused one has both
+    const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
+    if (!fc.flags && pad) {                          // uniform: before any barrier or TMEM use
+        if (threadIdx.x == 0) atomicOr(p.err, kErrBounds);
+        return;
+    }
+    uint8_t* smem = smem_raw + pad;
     const uint32_t sb = smem_u32(smem);
     auto V4 = [&](uint32_t off) -> uint4& { return *reinterpret_cast<uint4*>(smem + off); };
     constexpr uint32_t oKQ = G::OFF_KQ, oV = G::OFF_V, oXG = G::OFF_XG, oX = G::OFF_X;
@@ -262,8 +306,10 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + G::OFF_BAR);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + G::OFF_BAR + 8);
     const uint32_t mbar = smem_u32(bar);
-    __shared__ float gs[C], bs[C], Gs[C], g2[C];
-    __shared__ volatile int abort_flag;
+    float* Gs = reinterpret_cast<float*>(smem + G::OFF_G);
+    float* bs = Gs + C;
+    float* g2 = bs + C;
+    volatile int& abort_flag = *reinterpret_cast<volatile int*>(smem + G::OFF_BAR + 12);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q4 = warp & 3, cq = warp >> 2;         // TMEM lane quarter, column quarter
@@ -279,7 +325,7 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc(smem_u32(tmem_slot), 512);
+        tmem_alloc(smem_u32(tmem_slot), G::T_COLS);
         tmem_relinquish();
     }
     grid_dependency_wait();                          // the chunk inputs may come from the previous grid
@@ -304,7 +350,7 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
     // ---- loads (every global load issued before the shared stores)
     {
         constexpr int NKQ = 128 * (DK / 8) / kPrepThreads;
-        constexpr int NV = C * (DVP / 8) / kPrepThreads;
+        constexpr int NV = C * (DVMAX / 8) / kPrepThreads;
         uint4 kq[NKQ], vv[NV];
 #pragma unroll
         for (int u = 0; u < NKQ; ++u) {
@@ -347,8 +393,8 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
                 if (tid >= o) { x0 += y0; x1 += y1; }
             }
             x1 += __shfl_sync(0xffffffffu, x0, 31);
-            gs[tid] = x0;
-            gs[tid + 32] = x1;
+            Gs[tid] = x0;                             // log G, until warp 1 has replaced it below
+            Gs[tid + 32] = x1;
             bs[tid] = b0;
             bs[tid + 32] = b1;
         }
@@ -358,13 +404,19 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    if (tid < C) {
-        Gs[tid] = expf(gs[tid]);
-        g2[tid] = gs[tid] * 1.4426950408889634f;          // log2 domain for the decays
+    if (warp == 1) {
+        // beside the first MMAs' issue: G, log2 G, and the record's w, G_C
+        const float x0 = Gs[lane], x1 = Gs[lane + 32], gl = Gs[n - 1];
+        __syncwarp();
+        Gs[lane] = expf(x0);
+        Gs[lane + 32] = expf(x1);
+        g2[lane] = x0 * 1.4426950408889634f;          // log2 domain for the decays
+        g2[lane + 32] = x1 * 1.4426950408889634f;
         if (do_u) {
             float* misc = reinterpret_cast<float*>(rec + R::misc_off(dv));
-            misc[tid] = tid < n ? bs[tid] * expf(gs[n - 1] - gs[tid]) : 0.f;     // w_j
-            if (tid == 0) misc[C] = expf(gs[n - 1]);                            // G_C
+            misc[lane] = lane < n ? bs[lane] * expf(gl - x0) : 0.f;                              // w_j
+            misc[lane + 32] = lane + 32 < n ? bs[lane + 32] * expf(gl - x1) : 0.f;
+            if (lane == 0) misc[C] = expf(gl);                                                   // G_C
         }
     }
     bool ok = true;
@@ -416,9 +468,22 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
             y[c] = (keep && t < n) ? ex2(gt2 - g2[j]) * bs[j] * __uint_as_float(v[c]) : 0.f;
         }
         if (row < 64) {
-            float* dst = Lm + t * LSTRIDE + cq * 16;
+            // every lane writes its four 16-byte chunks in another order, so
+            // that neighbouring rows (a multiple of 32 banks apart) collide less
+            float4 v4[4];
 #pragma unroll
-            for (int j4 = 0; j4 < 16; j4 += 4) *reinterpret_cast<float4*>(dst + j4) = make_float4(y[j4], y[j4 + 1], y[j4 + 2], y[j4 + 3]);
+            for (int j = 0; j < 4; ++j) v4[j] = make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
+            auto rotate = [&](int by) {
+                float4 u4[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) u4[j] = v4[(j + by) & 3];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v4[j] = (lane & by) ? u4[j] : v4[j];
+            };
+            rotate(1);
+            rotate(2);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(Lm + t * LST + cq * 16 + 4 * ((j + lane) & 3)) = v4[j];
 #pragma unroll
             for (int c = 0; c < 16; ++c) y[c] = (cq * 16 + c == row) ? 1.f : 0.f;     // row of I
         }
@@ -437,21 +502,21 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
     // inverse of diagonal block j), row p of T solves x (I + L) = e_p column
     // block by column block from the right: x_j = (b_j - sum_{i > j} x_i L_ij) D_j,
     // zero right of column p.  The D_j come first (thread t < 64 solves
-    // column t mod 16 of block t / 16).
-    float* Dm = reinterpret_cast<float*>(smem + G::OFF_D);
+    // column t mod 16 of block t / 16) and take the places of L's diagonal
+    // blocks, which nothing else reads.
     if (ok && tid < 64) {
         const int kb = tid >> 4, c = tid & 15;
         float d[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const float* li = Lm + (16 * kb + i) * LSTRIDE + 16 * kb;
             float v = (i == c) ? 1.f : 0.f;
 #pragma unroll
-            for (int m = 0; m < i; ++m) v = fmaf(-li[m], d[m], v);
+            for (int m = 0; m < i; ++m) v = fmaf(-Lm[(16 * kb + i) * LST + 16 * kb + m], d[m], v);
             d[i] = v;
         }
+        __syncwarp();                                // a block's 16 threads share a warp
 #pragma unroll
-        for (int i = 0; i < 16; ++i) Dm[(16 * kb + i) * DSTRIDE + c] = d[i];
+        for (int i = 0; i < 16; ++i) Lm[(16 * kb + i) * LST + 16 * kb + c] = d[i];
     }
     __syncthreads();
     // Eight threads per row pr (tid = 8 pr + q); thread q owns columns
@@ -484,7 +549,7 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
             for (int o = 0; o < 8; ++o)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const float2 d2 = *reinterpret_cast<const float2*>(Dm + (16 * jb + 2 * (q ^ o) + e) * DSTRIDE + 2 * q);
+                    const float2 d2 = *reinterpret_cast<const float2*>(Lm + (16 * jb + 2 * (q ^ o) + e) * LST + 16 * jb + 2 * q);
                     xb[0] = fmaf(yv[o][e], d2.x, xb[0]);
                     xb[1] = fmaf(yv[o][e], d2.y, xb[1]);
                 }
@@ -503,7 +568,7 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const float2 l2 = *reinterpret_cast<const float2*>(
-                            Lm + (16 * jb + 2 * (q ^ o) + e) * LSTRIDE + 16 * kb + 2 * q);
+                            Lm + (16 * jb + 2 * (q ^ o) + e) * LST + 16 * kb + 2 * q);
                         xs[2 * kb + 0] = fmaf(-xv[o][e], l2.x, xs[2 * kb + 0]);
                         xs[2 * kb + 1] = fmaf(-xv[o][e], l2.y, xs[2 * kb + 1]);
                     }
@@ -599,7 +664,6 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
         const int t = row & 63;
         const float gt = Gs[t];
         const uint32_t oWQ = G::OFF_STAGE_WQ;
-        float* us = reinterpret_cast<float*>(smem + G::OFF_STAGE_U);
         const int n_w = do_w ? DK / 64 : 0;
         const int n_u = do_u ? (dv + 63) / 64 : 0;
         for (int k = 0; k < n_w + n_u; ++k) {            // uniform per block
@@ -637,15 +701,19 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
             } else if (ok) {
                 const int rc = 64 * (k - n_w) + 16 * cq;
                 if (rc < dv) {                           // uniform per warp
+                    float* us = reinterpret_cast<float*>(smem + (k == n_w ? G::OFF_STAGE_U0 : G::OFF_STAGE_U1));
                     uint32_t v[16];
                     tmem_ld16(tmem + lane_off + G::T_WU + DK + rc, v);
                     tmem_ld_wait();
 #pragma unroll
                     for (int j4 = 0; j4 < 16; j4 += 4)
-                        *reinterpret_cast<uint4*>(us + uau_idx(row, rc + j4)) = make_uint4(v[j4], v[j4 + 1], v[j4 + 2], v[j4 + 3]);
+                        *reinterpret_cast<uint4*>(us + uau_idx(row, 16 * cq + j4)) = make_uint4(v[j4], v[j4 + 1], v[j4 + 2], v[j4 + 3]);
                 }
             }
             fence_proxy_async_smem();
+            // the next piece is staged over what earlier stores read (the K
+            // image, [W; Q'])
+            if (PER_SM == 2 && tid == 0 && do_w && do_u && (k == n_w - 1 || k == n_w)) bulk_wait_read();
             __syncthreads();
             if (ok && tid == 0) {
                 if (w_piece) {
@@ -655,7 +723,7 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
                     const int u = k - n_w;                 // slices 2u, 2u + 1
                     const int slices = min(2, dv / 32 - 2 * u);
                     bulk_store(rec + R::uau_off() + (int64_t)u * 2 * (128 * 32 * 4),
-                               sb + G::OFF_STAGE_U + u * 2 * (128 * 32 * 4), slices * (128 * 32 * 4));
+                               sb + (u == 0 ? G::OFF_STAGE_U0 : G::OFF_STAGE_U1), slices * (128 * 32 * 4));
                 }
                 bulk_commit();
             }
@@ -686,19 +754,19 @@ __device__ __forceinline__ void gdn_prep_run(const GdnParams& p, const FuseCtl& 
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(*tmem_slot, 512);
+        tmem_dealloc(*tmem_slot, G::T_COLS);
     }
 }
 
-template <int DK>
-__global__ void __launch_bounds__(kPrepThreads, 1) gdn_prep_kernel(const __grid_constant__ GdnParams p) {
-    gdn_prep_run<DK>(p, FuseCtl{nullptr, 0}, blockIdx.x, gridDim.x);
+template <int DK, int PER_SM>
+__global__ void __launch_bounds__(kPrepThreads, PER_SM) gdn_prep_kernel(const __grid_constant__ GdnParams p) {
+    gdn_prep_run<DK, PER_SM>(p, FuseCtl{nullptr, 0}, blockIdx.x, gridDim.x);
 }
 
 // v2 prep: the front (loads .. [W | U]) is the v1 prep's; the record differs.
 template <int DK>
 __device__ __forceinline__ void gdn_prep2_run(const GdnParams& p, const FuseCtl& fc, int u0, int ustride) {
-    using G = PrepCfg<DK>;
+    using G = PrepWide<DK>;
     using G2 = Prep2Cfg<DK>;
     using R = Rec2<DK>;
     extern __shared__ uint8_t smem_raw[];
@@ -1761,7 +1829,7 @@ __global__ void __launch_bounds__(kThreads, 1) gdn_scan_kernel(const __grid_cons
 // the (chunk, head) units in fused_unit order and publish each record through
 // its flag.  A scan waits only for records, and prep workers never wait, so
 // the launch completes as long as every prep worker eventually gets an SM:
-// the scan items leave at least kMinPrepWorkers SMs, other kernels' blocks
+// the scan items leave two thirds of the SMs, other kernels' blocks
 // (the compaction beside it) finish on their own, and the kernels after it
 // on the stream cannot take an SM before every block of it has started
 // (their launch waits for every block's launch_dependents).  Not a
@@ -1777,7 +1845,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) gdn_fused_kernel(const __grid
         const int slices = p.dv / p.dv_slice;
         gdn_scan_packed_run<DK>(p, fc, x / (slices * p.H), (x / slices) % p.H, (x % slices) * p.dv_slice);
     } else {
-        gdn_prep_run<DK>(p, fc, x - p.n_scan, gridDim.x - p.n_scan);
+        gdn_prep_run<DK, 1>(p, fc, x - p.n_scan, gridDim.x - p.n_scan);
     }
 }
 
@@ -2151,8 +2219,18 @@ void configure_once(int smem) {
 
 template <int DK>
 void launch_prep_dk(const GdnParams& p, cudaStream_t s) {
-    configure_once<gdn_prep_kernel<DK>>(PrepCfg<DK>::SMEM);
-    launch_pdl(gdn_prep_kernel<DK>, dim3(p.total_chunks * p.H * p.prep_parts), dim3(kPrepThreads), PrepCfg<DK>::SMEM, s, p);
+    // two blocks an SM (64 registers a thread) once a block each does not
+    // cover the grid: 2464 units (32 characters' tails) 222 -> 153 us, a
+    // 1024-token layer of 16 heads 56.7 -> 50.7; with few blocks the one-block
+    // form is faster (a 64-token layer 14.0 against 14.6)
+    const int grid = p.total_chunks * p.H * p.prep_parts;
+    if (grid > p.num_sms) {
+        configure_once<gdn_prep_kernel<DK, 2>>(PrepCfg<DK, 2>::SMEM);
+        launch_pdl(gdn_prep_kernel<DK, 2>, dim3(grid), dim3(kPrepThreads), PrepCfg<DK, 2>::SMEM, s, p);
+    } else {
+        configure_once<gdn_prep_kernel<DK, 1>>(PrepCfg<DK, 1>::SMEM);
+        launch_pdl(gdn_prep_kernel<DK, 1>, dim3(grid), dim3(kPrepThreads), PrepCfg<DK, 1>::SMEM, s, p);
+    }
 }
 
 template <int DK, int CW>
@@ -2170,7 +2248,7 @@ void launch_scan_dk(const GdnParams& p, cudaStream_t s) {
 
 template <int DK>
 cudaError_t launch_fused_dk(const GdnParams& p, int grid, cudaStream_t s) {
-    constexpr int smem = ScanCfg<DK>::SMEM > PrepCfg<DK>::SMEM ? ScanCfg<DK>::SMEM : PrepCfg<DK>::SMEM;
+    constexpr int smem = std::max(ScanCfg<DK>::SMEM, PrepCfg<DK, 1>::SMEM + 1024);
     configure_once<gdn_fused_kernel<DK, 16>>(smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -2187,7 +2265,7 @@ cudaError_t launch_fused_dk(const GdnParams& p, int grid, cudaStream_t s) {
 
 template <int DK>
 void launch_v2_dk(const GdnParams& p, int fused_grid, cudaStream_t s, cudaError_t* fused_err) {
-    constexpr int fsmem = Chain2Cfg<DK>::SMEM > PrepCfg<DK>::SMEM ? Chain2Cfg<DK>::SMEM : PrepCfg<DK>::SMEM;
+    constexpr int fsmem = Chain2Cfg<DK>::SMEM > PrepWide<DK>::SMEM ? Chain2Cfg<DK>::SMEM : PrepWide<DK>::SMEM;
     if (fused_grid > 0) {
         configure_once<gdn_fused2_kernel<DK>>(fsmem);
         cudaLaunchConfig_t cfg = {};
@@ -2205,8 +2283,8 @@ void launch_v2_dk(const GdnParams& p, int fused_grid, cudaStream_t s, cudaError_
         *fused_err = cudaLaunchKernelEx(&cfg, gdn_fused2_kernel<DK>, p);
         if (*fused_err != cudaSuccess) return;
     } else {
-        configure_once<gdn_prep2_kernel<DK>>(PrepCfg<DK>::SMEM);
-        launch_pdl(gdn_prep2_kernel<DK>, dim3(p.total_chunks * p.H), dim3(kPrepThreads), PrepCfg<DK>::SMEM, s, p);
+        configure_once<gdn_prep2_kernel<DK>>(PrepWide<DK>::SMEM);
+        launch_pdl(gdn_prep2_kernel<DK>, dim3(p.total_chunks * p.H), dim3(kPrepThreads), PrepWide<DK>::SMEM, s, p);
         configure_once<gdn_chain2_kernel<DK>>(Chain2Cfg<DK>::SMEM);
         launch_pdl(gdn_chain2_kernel<DK>, dim3(p.dv / 32, p.H, p.n_chars), dim3(kThreads), Chain2Cfg<DK>::SMEM, s, p);
     }

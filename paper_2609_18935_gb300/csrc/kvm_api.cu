@@ -66,7 +66,6 @@ constexpr int kFlagStride = 32;     // compaction read flags: one per 128-byte l
 // tokens 14 : 12.7 and 21 : 18 for 1 and 8.
 constexpr int recur_tail(int dk) { return dk == 64 ? 48 : 32; }
 constexpr int kRecurTile = 16;      // tokens it stages at a time when blocks share an SM
-constexpr int kMinPrepWorkers = 24; // fused delta-rule launches leave at least this many SMs to the prep
 
 }  // namespace
 
@@ -1270,17 +1269,19 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     // two prep blocks per (chunk, head) when both fit on the SMs at once: they
     // share the solve for X and halve the products, staging and record
     // stores that follow it
+    p.num_sms = c->num_sms;
     p.prep_parts = (int64_t)2 * chunks * c->H <= c->num_sms ? 2 : 1;
-    // One launch for both when the scan items leave enough SMs to prep
-    // workers (few characters) and the prep needs several rounds of them
-    // (long tails): the chunk scan then starts on the first records while
-    // the prep still works on later chunks.  Measured in a stack of
-    // delta-rule layers (pipelined launches): 59.6 against 62.3 us a layer
-    // for a 1024-token tail, but 27.0 against 22.4 us for 256 tokens, whose
-    // prep is a single wave either way.  Otherwise the prep grid, then the scan.
+    // One launch for both when the scan items leave most SMs to prep workers
+    // (few characters) and the prep is more than one wave of two blocks an SM
+    // (long tails): the chunk scan then starts on the first records while the
+    // prep still works on later chunks.  Fused against two launches, us a layer:
+    // 104 workers (12 heads of 128) 89 : 94 at 2048 tokens, 169 : 181 at 4096;
+    // 120 workers (d_k 64) 77 : 88, 154 : 166; but 88 workers (16 heads of 128)
+    // 53 : 51 at 1024 and 203 : 198 at 4096, 24 workers (32 heads) 309 : 76 at
+    // 1024.  Otherwise the prep grid, then the scan.
     const int items = c->B * c->H * (c->dv / p.dv_slice);
     const int workers = c->num_sms - items;
-    const bool fuse = c->gdn_fuse && p.dv_slice <= 32 && workers >= kMinPrepWorkers && chunks * c->H >= 2 * workers;
+    const bool fuse = c->gdn_fuse && p.dv_slice <= 32 && 3 * workers >= 2 * c->num_sms && chunks * c->H > 2 * c->num_sms;
     if (c->gdn_chain && c->gdn_snap && p.dv_slice == 32) {
         // state-chain form: the chain carries only S (one MMA batch a chunk),
         // the outputs follow in a parallel pass over per-chunk snapshots
