@@ -11,228 +11,252 @@
 //
 //  probe_rotate : rotate the caller's probe queries (fp64 angle reduced mod
 //                 2 pi, fp32 rotation) into an fp32 workspace;
-//  probe_tiles  : (pass A) per 64-key tile and query row, the tile's max
-//                 score and sum of exp(s - max);
-//  probe_rows   : per query row, the softmax max and denominator from the
-//                 tiles' partials;
-//  probe_tiles  : (pass C) the scores again, p = exp(s - max) / sum, summed
-//                 over every query row: the averaged distribution of each
-//                 key, and its group's mass (atomic adds) when groups are
-//                 given.
-// This is a diagnostic, not the hot path: fp32 on the CUDA cores, scores
-// recomputed in pass C rather than stored.
+//  probe_scores : S = Q K^T of 64 rows (query, head of the group) of one KV
+//                 head and 64 keys a block, in fp32 on the CUDA cores;
+//  probe_rows   : per row, the softmax max and one over the denominator;
+//  probe_probs  : p = exp(s - max) / sum summed over the rows: the averaged
+//                 distribution of each key, and its group's mass (atomic adds)
+//                 when groups are given.
+//
+// The scores are formed once and pass through memory (the attention's partials
+// workspace; row blocks that do not fit together are done in turn).  8192 keys,
+// 8 queries of 16 heads of 256 (0.54 GFLOP): rotate 4, scores 22,
+// rows 5, probs 13 us alone, 61 together, against 210 with the scores formed
+// twice by 128 threads a tile and one thread a row merging the tiles
+// Fp32 products throughout: on the tensor cores the queries would have to be
+// split, and this is the reference that other paths are judged by.
+#include <algorithm>
+
 #include "kvm_internal.cuh"
 
 namespace kvm {
 namespace {
 
 constexpr double kTwoPiP = 6.283185307179586476925286766559;
-constexpr int kProbeThreads = 256;
-constexpr int kRowChunk = 64;                  // query rows staged per step
-constexpr int kRowsPerThread = kRowChunk / (kProbeThreads / kProbeKeys);   // 16
+constexpr int kScoreThreads = 128;
+constexpr int kDims = 32;                      // dims staged per step
+constexpr int kPitch = 64 + 4;                 // row pitch of the staged [dim][64] tiles
+constexpr int kProbThreads = 256;              // probe_probs: 32 keys, eight threads each
 
+using f2 = unsigned long long;                 // two packed floats
+
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// One block per (query, head).
 __global__ void __launch_bounds__(128) probe_rotate_kernel(const __grid_constant__ ProbeParams p) {
     grid_dependency_wait();
     grid_dependents_launch();
-    const int i = blockIdx.x;
+    const int i = blockIdx.x / p.Hq, half = p.R / 2;
     const int64_t pos = p.pos[p.slot0 + p.L - p.n_q + i];
-    const int half = p.R / 2;
-    __shared__ float cs[kMaxRotaryHalf], sn[kMaxRotaryHalf];
+    const __nv_bfloat16* q = p.q + (int64_t)blockIdx.x * p.D;
+    float* o = p.q_rot + (int64_t)blockIdx.x * p.D;
     for (int d = threadIdx.x; d < half; d += blockDim.x) {
         const double ang = (double)pos * p.inv_freq[d];
         const double r = fma(-rint(ang * (1.0 / kTwoPiP)), kTwoPiP, ang);
-        float sv, cv;
-        sincosf((float)r, &sv, &cv);
-        cs[d] = cv;
-        sn[d] = sv;
+        float sn, cs;
+        sincosf((float)r, &sn, &cs);
+        const float x = __bfloat162float(q[d]), y = __bfloat162float(q[d + half]);
+        o[d] = x * cs - y * sn;
+        o[d + half] = y * cs + x * sn;
     }
-    __syncthreads();
-    const __nv_bfloat16* q = p.q + (int64_t)i * p.Hq * p.D;
-    float* o = p.q_rot + (int64_t)i * p.Hq * p.D;
-    for (int idx = threadIdx.x; idx < p.Hq * p.D; idx += blockDim.x) {
-        const int d = idx % p.D, row = idx - d;
-        const float x = __bfloat162float(q[idx]);
-        float y = x;
-        if (d < half) y = x * cs[d] - __bfloat162float(q[row + d + half]) * sn[d];
-        else if (d < p.R) y = x * cs[d - half] + __bfloat162float(q[row + d - half]) * sn[d - half];
-        o[idx] = y;
-    }
+    for (int d = p.R + threadIdx.x; d < p.D; d += blockDim.x) o[d] = __bfloat162float(q[d]);
 }
 
-// Shared memory: the key tile of one KV head [64][D + 2] bf16 (the pad makes
-// the row stride an odd number of words, so lanes reading different keys at
-// the same column hit different banks), then a chunk of query rows
-// [64][D] fp32 (read as broadcasts), then the reduction scratch.
-template <bool kFinal>
-__global__ void __launch_bounds__(kProbeThreads) probe_tiles_kernel(const __grid_constant__ ProbeParams p) {
+// grid (key tiles, row blocks).  Thread (ty, tx) forms rows 8 ty .. + 7 (in
+// packed pairs) and keys 4 tx .. + 3 of the 64 x 64 tile; q and k are staged
+// 32 dims at a time as [dim][64].  Row rg of KV head kv is query rg / g, head
+// kv g + rg mod g.
+__global__ void __launch_bounds__(kScoreThreads) probe_scores_kernel(const __grid_constant__ ProbeParams p) {
+    __shared__ __align__(16) float Qs[kDims][kPitch], Ks[kDims][kPitch];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int rows_kv = p.n_q * p.g, blocks_kv = (rows_kv + kProbeRows - 1) / kProbeRows;
+    const int rb = p.row_block0 + blockIdx.y;
+    const int kv = rb / blocks_kv, r0 = (rb % blocks_kv) * kProbeRows;
+    const int D = p.D, j0 = blockIdx.x * kProbeKeys;
     grid_dependency_wait();
     grid_dependents_launch();
-    extern __shared__ __align__(16) uint8_t smem[];
-    const int D = p.D, KS = D / 2 + 1;                     // key row stride in 32-bit words
-    uint32_t* Ks = reinterpret_cast<uint32_t*>(smem);
-    float* Qs = reinterpret_cast<float*>(smem + (size_t)kProbeKeys * KS * 4);
-    float* red = Qs + (size_t)kRowChunk * D;                // [rsub][half][rows][2] = 4 * 2 * 16 * 2
-    float* acc_s = red + 4 * 2 * kRowsPerThread * 2;        // [4][64] per-key partial sums (pass C)
-    const int t = threadIdx.x;
-    const int kk = t & (kProbeKeys - 1), rsub = t / kProbeKeys, whalf = kk >> 5;
-    const int tile = blockIdx.x;
-    const int j = tile * kProbeKeys + kk;                   // this thread's key (live index)
-    const int rows_kv = p.n_q * p.g;
-    const int n_rows = p.n_q * p.Hq;
-    const int first_q = p.L - p.n_q;                        // live index of probe query 0
-    float acc = 0.f;
-
-    for (int kv = 0; kv < p.Hkv; ++kv) {
-        __syncthreads();                                    // the previous key tile is consumed
-        const __nv_bfloat16* kb = p.K + ((int64_t)kv * p.slab_rows + p.slot0 + (int64_t)tile * kProbeKeys) * D;
-        for (int idx = t; idx < kProbeKeys * (D / 2); idx += kProbeThreads) {
-            const int r = idx / (D / 2), w = idx % (D / 2);
-            const bool in = tile * kProbeKeys + r < p.L;
-            Ks[r * KS + w] = in ? reinterpret_cast<const uint32_t*>(kb + (int64_t)r * D)[w] : 0u;
-        }
-        for (int c0 = 0; c0 < rows_kv; c0 += kRowChunk) {
-            __syncthreads();                                // the previous query chunk is consumed
-            for (int idx = t; idx < kRowChunk * D; idx += kProbeThreads) {
-                const int r = idx / D, d = idx % D, rg = c0 + r;
-                float v = 0.f;
-                if (rg < rows_kv) {
-                    const int i = rg / p.g, h = kv * p.g + rg % p.g;
-                    v = p.q_rot[((int64_t)i * p.Hq + h) * D + d];
-                }
-                Qs[idx] = v;
-            }
-            __syncthreads();
-            float s[kRowsPerThread];
+    const __nv_bfloat16* kb = p.K + ((int64_t)kv * p.slab_rows + p.slot0 + j0) * D;
+    // staging: thread t moves dims 8 (t mod 4) .. + 7 of tile rows t / 4, t / 4 + 32
+    const int c = (tid & 3) * 8, sr = tid >> 2;
+    const float* qr[2];
+    bool q_in[2], k_in[2];
 #pragma unroll
-            for (int r = 0; r < kRowsPerThread; ++r) s[r] = 0.f;
-            const uint32_t* krow = Ks + kk * KS;
-            const float* qb = Qs + (size_t)(rsub * kRowsPerThread) * D;
-            for (int w = 0; w < D / 2; ++w) {
-                const uint32_t kw = krow[w];
-                const float k0 = __uint_as_float(kw << 16), k1 = __uint_as_float(kw & 0xffff0000u);
-#pragma unroll
-                for (int r = 0; r < kRowsPerThread; ++r) {
-                    const float2 q2 = *reinterpret_cast<const float2*>(qb + (size_t)r * D + 2 * w);
-                    s[r] = fmaf(q2.x, k0, fmaf(q2.y, k1, s[r]));
-                }
-            }
-            // mask: rows past the end, keys past the row's causal limit
-#pragma unroll
-            for (int r = 0; r < kRowsPerThread; ++r) {
-                const int rg = c0 + rsub * kRowsPerThread + r;
-                const int i = rg / p.g;
-                const bool vis = rg < rows_kv && j < p.L && j <= first_q + i;
-                s[r] = vis ? s[r] * p.scale : -INFINITY;
-            }
-            if (!kFinal) {
-                // per row: this warp's (max, sum over its 32 keys), then the
-                // two warps of the row group combine
-#pragma unroll
-                for (int r = 0; r < kRowsPerThread; ++r) {
-                    float m = s[r];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                    float e = (m == -INFINITY) ? 0.f : expf(s[r] - m);
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-                    if ((t & 31) == 0) {
-                        red[((rsub * 2 + whalf) * kRowsPerThread + r) * 2 + 0] = m;
-                        red[((rsub * 2 + whalf) * kRowsPerThread + r) * 2 + 1] = e;
-                    }
-                }
-                __syncthreads();
-                if (kk < kRowsPerThread) {                  // one thread per (rsub, row)
-                    const int r = kk;
-                    const int rg = c0 + rsub * kRowsPerThread + r;
-                    if (rg < rows_kv) {
-                        const float m0 = red[((rsub * 2 + 0) * kRowsPerThread + r) * 2 + 0];
-                        const float e0 = red[((rsub * 2 + 0) * kRowsPerThread + r) * 2 + 1];
-                        const float m1 = red[((rsub * 2 + 1) * kRowsPerThread + r) * 2 + 0];
-                        const float e1 = red[((rsub * 2 + 1) * kRowsPerThread + r) * 2 + 1];
-                        const float m = fmaxf(m0, m1);
-                        const float e = (m == -INFINITY) ? 0.f : e0 * expf(m0 - m) + e1 * expf(m1 - m);
-                        const int row = (rg / p.g) * p.Hq + kv * p.g + rg % p.g;
-                        p.part[((int64_t)tile * n_rows + row) * 2 + 0] = m;
-                        p.part[((int64_t)tile * n_rows + row) * 2 + 1] = e;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int r = 0; r < kRowsPerThread; ++r) {
-                    const int rg = c0 + rsub * kRowsPerThread + r;
-                    if (rg < rows_kv && s[r] != -INFINITY) {
-                        const int row = (rg / p.g) * p.Hq + kv * p.g + rg % p.g;
-                        const float m = p.row_ms[2 * row], den = p.row_ms[2 * row + 1];
-                        acc += expf(s[r] - m) / den;
-                    }
-                }
-            }
-        }
+    for (int i = 0; i < 2; ++i) {
+        const int rg = r0 + sr + 32 * i;
+        q_in[i] = rg < rows_kv;
+        qr[i] = p.q_rot + (q_in[i] ? ((int64_t)(rg / p.g) * p.Hq + kv * p.g + rg % p.g) * D : 0);
+        k_in[i] = j0 + sr + 32 * i < p.L;
     }
-    if (kFinal) {
-        acc_s[rsub * kProbeKeys + kk] = acc;
+    uint4 kx[2];
+    float4 qx[2][2];
+    auto load = [&](int d) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            kx[i] = k_in[i] ? *reinterpret_cast<const uint4*>(kb + (int64_t)(sr + 32 * i) * D + d + c) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                qx[i][e] = q_in[i] ? *reinterpret_cast<const float4*>(qr[i] + d + c + 4 * e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    f2 acc[4][4];                                             // [row pair][key]
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0;
+    load(0);
+    for (int d0 = 0; d0 < D; d0 += kDims) {
+        __syncthreads();                                      // the previous step is consumed
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t* w = reinterpret_cast<const uint32_t*>(&kx[i]);
+            const float* f = reinterpret_cast<const float*>(&qx[i][0]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                Ks[c + 2 * e][sr + 32 * i] = __uint_as_float(w[e] << 16);
+                Ks[c + 2 * e + 1][sr + 32 * i] = __uint_as_float(w[e] & 0xffff0000u);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) Qs[c + e][sr + 32 * i] = f[e];
+        }
         __syncthreads();
-        if (rsub == 0 && j < p.L) {
-            const float tot = (acc_s[kk] + acc_s[kProbeKeys + kk] + acc_s[2 * kProbeKeys + kk] +
-                               acc_s[3 * kProbeKeys + kk]) / (float)n_rows;
-            p.probs[j] = tot;
-            if (p.group_of) {
-                const int gid = p.group_of[j];
-                if (gid >= p.n_groups) atomicOr(p.err, kErrBounds);
-                else if (gid >= 0) atomicAdd(p.group_mass + gid, tot);
-            }
+        if (d0 + kDims < D) load(d0 + kDims);                 // in flight during the products
+#pragma unroll 8
+        for (int d = 0; d < kDims; ++d) {
+            const float4 k4 = *reinterpret_cast<const float4*>(&Ks[d][4 * tx]);
+            const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&Qs[d][8 * ty]);
+            const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(&Qs[d][8 * ty + 4]);
+            const f2 kk[4] = {pack2(k4.x, k4.x), pack2(k4.y, k4.y), pack2(k4.z, k4.z), pack2(k4.w, k4.w)};
+            const f2 qq[4] = {qa.x, qa.y, qb.x, qb.y};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) acc[a][b] = fma2(qq[a], kk[b], acc[a][b]);
         }
     }
+    // rows past the end, keys past the row's causal limit: -inf
+    const int j = j0 + 4 * tx, first_q = p.L - p.n_q;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+        const int r = 8 * ty + a, rg = r0 + r, lim = rg < rows_kv ? first_q + rg / p.g : -1;
+        float s[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const float2 x = unpack2(acc[a >> 1][b]);
+            s[b] = j + b <= lim ? (a & 1 ? x.y : x.x) * p.scale : -INFINITY;
+        }
+        if (j < p.pitch)
+            *reinterpret_cast<float4*>(p.scores + ((int64_t)blockIdx.y * kProbeRows + r) * p.pitch + j) =
+                make_float4(s[0], s[1], s[2], s[3]);
+    }
 }
 
-__global__ void probe_rows_kernel(const __grid_constant__ ProbeParams p) {
+// One block per row of the staged row blocks (rows past a head's end have no
+// key: max -inf, factor 0).
+__global__ void __launch_bounds__(256) probe_rows_kernel(const __grid_constant__ ProbeParams p) {
     grid_dependency_wait();
     grid_dependents_launch();
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n_rows = p.n_q * p.Hq;
-    if (row >= n_rows) return;
-    const int tiles = (p.L + kProbeKeys - 1) / kProbeKeys;
-    float m = -INFINITY, e = 0.f;
-    for (int tl = 0; tl < tiles; ++tl) {
-        const float mt = p.part[((int64_t)tl * n_rows + row) * 2 + 0];
-        const float et = p.part[((int64_t)tl * n_rows + row) * 2 + 1];
-        if (mt == -INFINITY) continue;
-        const float nm = fmaxf(m, mt);
-        e = (m == -INFINITY ? 0.f : e * expf(m - nm)) + et * expf(mt - nm);
-        m = nm;
+    __shared__ float red[8];
+    const float4* s = reinterpret_cast<const float4*>(p.scores + (int64_t)blockIdx.x * p.pitch);
+    const int n4 = p.pitch / 4, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float m = -INFINITY;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < n4; k += 256) {
+        const float4 x = s[k];
+        m = fmaxf(m, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
     }
-    p.row_ms[2 * row] = m;
-    p.row_ms[2 * row + 1] = e;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) red[warp] = m;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m = fmaxf(m, red[k]);
+    __syncthreads();
+    float e = 0.f;
+    if (m != -INFINITY) {
+#pragma unroll 4
+        for (int k = threadIdx.x; k < n4; k += 256) {
+            const float4 x = s[k];
+            e += (expf(x.x - m) + expf(x.y - m)) + (expf(x.z - m) + expf(x.w - m));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (lane == 0) red[warp] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        e = 0.f;
+        for (int k = 0; k < 8; ++k) e += red[k];
+        p.row_ms[2 * blockIdx.x] = m;
+        p.row_ms[2 * blockIdx.x + 1] = m == -INFINITY ? 0.f : 1.f / e;
+    }
 }
 
-size_t probe_smem(int D) {
-    return (size_t)kProbeKeys * (D / 2 + 1) * 4 + (size_t)kRowChunk * D * 4 + 4 * 2 * kRowsPerThread * 2 * 4 +
-           4 * kProbeKeys * 4;
-}
-
-template <auto KERNEL>
-void probe_configure(size_t smem) {
-    static unsigned long long configured = 0;   // one bit per device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (!(configured >> (dev & 63) & 1ull)) {
-        cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        configured |= 1ull << (dev & 63);
+// 32 keys a block, warp w taking every eighth row.  Row blocks done in turn
+// add up in probs_out; the last one scales and adds the group masses.
+__global__ void __launch_bounds__(kProbThreads) probe_probs_kernel(const __grid_constant__ ProbeParams p) {
+    grid_dependency_wait();
+    grid_dependents_launch();
+    __shared__ float part[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int j = blockIdx.x * 32 + lane, n = p.n_row_blocks * kProbeRows;
+    float acc = 0.f;
+    if (j < p.L) {
+#pragma unroll 8
+        for (int r = w; r < n; r += 8) {
+            const float2 ms = *reinterpret_cast<const float2*>(p.row_ms + 2 * r);
+            const float s = p.scores[(int64_t)r * p.pitch + j];
+            acc += s == -INFINITY ? 0.f : expf(s - ms.x) * ms.y;
+        }
+    }
+    part[w][lane] = acc;
+    __syncthreads();
+    if (w > 0 || j >= p.L) return;
+    float tot = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) tot += part[k][lane];
+    if (p.row_block0 > 0) tot += p.probs[j];
+    if (p.last) tot /= (float)(p.n_q * p.Hq);
+    p.probs[j] = tot;
+    if (p.last && p.group_of) {
+        const int gid = p.group_of[j];
+        if (gid >= p.n_groups) atomicOr(p.err, kErrBounds);
+        else if (gid >= 0) atomicAdd(p.group_mass + gid, tot);
     }
 }
 
 }  // namespace
 
-void launch_attn_probe(const ProbeParams& p, cudaStream_t s) {
-    if (p.L <= 0 || p.n_q <= 0) return;
-    const int tiles = (p.L + kProbeKeys - 1) / kProbeKeys;
-    const size_t smem = probe_smem(p.D);
-    probe_configure<probe_tiles_kernel<false>>(smem);
-    probe_configure<probe_tiles_kernel<true>>(smem);
-    launch_pdl(probe_rotate_kernel, dim3(p.n_q), dim3(128), 0, s, p);
-    launch_pdl(probe_tiles_kernel<false>, dim3(tiles), dim3(kProbeThreads), smem, s, p);
-    launch_pdl(probe_rows_kernel, dim3((p.n_q * p.Hq + 127) / 128), dim3(128), 0, s, p);
-    launch_pdl(probe_tiles_kernel<true>, dim3(tiles), dim3(kProbeThreads), smem, s, p);
+int probe_row_blocks(int n_q, int Hkv, int g) { return Hkv * ((n_q * g + kProbeRows - 1) / kProbeRows); }
+
+int launch_attn_probe(ProbeParams p, cudaStream_t s) {
+    if (p.L <= 0 || p.n_q <= 0) return 0;
+    const int tiles = (p.L + kProbeKeys - 1) / kProbeKeys, total = probe_row_blocks(p.n_q, p.Hkv, p.g);
+    p.pitch = (p.L + 3) / 4 * 4;
+    const int fit = (int)std::min<int64_t>(total, p.scores_cap / ((int64_t)kProbeRows * p.pitch));
+    launch_pdl(probe_rotate_kernel, dim3(p.n_q * p.Hq), dim3(128), 0, s, p);
+    int launches = 1;
+    for (p.row_block0 = 0; p.row_block0 < total; p.row_block0 += p.n_row_blocks, launches += 3) {
+        p.n_row_blocks = std::min(fit, total - p.row_block0);
+        p.last = p.row_block0 + p.n_row_blocks == total;
+        launch_pdl(probe_scores_kernel, dim3(tiles, p.n_row_blocks), dim3(kScoreThreads), 0, s, p);
+        launch_pdl(probe_rows_kernel, dim3(p.n_row_blocks * kProbeRows), dim3(256), 0, s, p);
+        launch_pdl(probe_probs_kernel, dim3((p.L + 31) / 32), dim3(kProbThreads), 0, s, p);
+    }
+    return launches;
 }
 
 }  // namespace kvm

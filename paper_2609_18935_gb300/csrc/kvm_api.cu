@@ -103,7 +103,7 @@ struct kvm_ctx {
     int32_t* pos_host = nullptr;          // pinned [max(max_tail, max capacity)]
     cudaEvent_t ev_pos = nullptr;
     int max_cap = 0;
-    // attention-probe workspace: rotated probe queries, per-tile and per-row softmax partials
+    // attention-probe workspace: rotated probe queries, per-row softmax max and factor
     // short convolution: weights [n_gdn][C][4] fp32; state, two buffers per
     // layer [2][n_gdn][B][3][C] bf16 (a round reads one, writes the other,
     // conv_par[layer] tells which is current); outputs [max_tail][H][...] bf16
@@ -112,9 +112,9 @@ struct kvm_ctx {
     std::vector<int> conv_par;
     __nv_bfloat16* conv_y = nullptr;
     float* probe_q = nullptr;
-    float* probe_part = nullptr;
     float* probe_rows = nullptr;
     float* part_o = nullptr;
+    size_t part_floats = 0;               // of part_o
     float* part_ml = nullptr;
     int32_t* tickets = nullptr;
     uint32_t* flags = nullptr;
@@ -536,13 +536,14 @@ extern "C" kvm_status kvm_create(const kvm_model_desc* m, int32_t n_chars, const
     }
     if (c->n_attn) {
         const size_t rows = (size_t)kProbeMaxQueries * c->Hq;
-        const size_t tiles = ((size_t)c->max_cap + kProbeKeys - 1) / kProbeKeys;
         if (e == cudaSuccess) e = alloc_zero(&c->probe_q, rows * c->D);
-        if (e == cudaSuccess) e = alloc_zero(&c->probe_part, tiles * rows * 2);
-        if (e == cudaSuccess) e = alloc_zero(&c->probe_rows, rows * 2);
+        if (e == cudaSuccess)
+            e = alloc_zero(&c->probe_rows, (size_t)probe_row_blocks(kProbeMaxQueries, c->Hkv, c->g) * kProbeRows * 2);
     }
     const size_t part_slots = c->n_attn ? 2 * (size_t)attention_grid_cap(c->num_sms, c->D) : 0;
-    if (e == cudaSuccess) e = alloc_zero(&c->part_o, part_slots * kAttnRows * c->D);
+    // the probe's scores share the partials' space: 64 rows of the longest character at least
+    c->part_floats = c->n_attn ? std::max(part_slots * kAttnRows * c->D, (size_t)kProbeRows * c->max_cap) : 0;
+    if (e == cudaSuccess) e = alloc_zero(&c->part_o, c->part_floats);
     if (e == cudaSuccess) e = alloc_zero(&c->part_ml, part_slots * kAttnRows * 2);
     if (e == cudaSuccess) e = alloc_zero(&c->tickets, (size_t)n_chars * (n_kv_slabs + 1));
     if (e == cudaSuccess) e = alloc_zero(&c->flags, n_flags * kFlagStride);
@@ -1453,7 +1454,8 @@ extern "C" kvm_status kvm_attn_probe(kvm_ctx* c, int32_t layer, int32_t b, int32
     p.q_rot = c->probe_q;
     p.K = c->K + (size_t)c->attn_idx[layer] * c->Hkv * c->T_cap * c->D;
     p.pos = c->pos;
-    p.part = c->probe_part;
+    p.scores = c->part_o;
+    p.scores_cap = (int64_t)c->part_floats;
     p.row_ms = c->probe_rows;
     p.probs = probs_out;
     p.group_of = group_of;
@@ -1461,8 +1463,7 @@ extern "C" kvm_status kvm_attn_probe(kvm_ctx* c, int32_t layer, int32_t b, int32
     p.err = c->err;
     for (int d = 0; d < c->R / 2; ++d) p.inv_freq[d] = c->inv_freq[d];
     if (group_of) CUDA_TRY(cudaMemsetAsync(group_mass_out, 0, sizeof(float) * (size_t)n_groups, s));
-    c->launches += 4;
-    launch_attn_probe(p, s);
+    c->launches += launch_attn_probe(p, s);
     LAUNCH_CHECK(c);
     return KVM_OK;
 }

@@ -199,7 +199,8 @@ constexpr int kAttnRows = 128;   // query rows per attention tile
 // attention-probe diagnostics (§5.3, Appendix C)
 // ----------------------------------------------------------------------------
 constexpr int kProbeMaxQueries = 16;   // probe queries per call (the paper averages the last 8)
-constexpr int kProbeKeys = 64;         // keys per probe block
+constexpr int kProbeKeys = 64;         // keys per score tile
+constexpr int kProbeRows = 64;         // query rows per score tile
 
 struct ProbeParams {
     int32_t L;            // live entries of the character
@@ -213,15 +214,20 @@ struct ProbeParams {
     float* q_rot;             // workspace [n_q][Hq][D] fp32
     const __nv_bfloat16* K;   // this layer's K slabs [Hkv][slab_rows][D]
     const int32_t* pos;       // [slab_rows]
-    float* part;              // workspace [ceil(L / 64)][n_q * Hq][2]: per key tile (max, sum)
-    float* row_ms;            // workspace [n_q * Hq][2]: per query row (max, sum)
+    float* scores;            // workspace [n_row_blocks * 64][pitch]
+    int64_t scores_cap;       // its floats; at least 64 rows of any character
+    int32_t pitch;            // L rounded up to 4
+    int32_t row_block0, n_row_blocks;   // 64-row blocks of this pass (each within one KV head)
+    int32_t last;             // the last pass
+    float* row_ms;            // workspace [n_row_blocks * 64][2]: per query row (max, 1 / sum)
     float* probs;             // out [L]
     const int32_t* group_of;  // [L] or null
     float* group_mass;        // out [n_groups]
     int32_t* err;
     double inv_freq[kMaxRotaryHalf];
 };
-void launch_attn_probe(const ProbeParams& p, cudaStream_t s);
+int probe_row_blocks(int n_q, int Hkv, int g);
+int launch_attn_probe(ProbeParams p, cudaStream_t s);   // returns the number of launches
 
 // ----------------------------------------------------------------------------
 // gated delta rule

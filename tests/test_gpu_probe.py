@@ -80,3 +80,29 @@ def test_probe_rejects_bad_requests():
         pair.ctx.attn_probe(1, 0, q, group_of=torch.full((20,), 3, dtype=torch.int32, device="cuda"), n_groups=2)
         pair.ctx.check()
     pair.ctx.check()
+
+
+@pytest.mark.parametrize("hq,hkv,head_dim,rotary,n_q,live,cap", [
+    (64, 1, 64, 64, 16, 1500, 60000),       # 1024 rows: more score rows than the workspace holds at once
+    (6 * 4, 6, 128, 30, 5, 131, 256),       # a rotary half that is no multiple of eight, ragged keys and rows
+    (2, 2, 256, 0, 1, 1, 128),              # a single key, no rotation
+])
+def test_probe_row_blocks_and_edges(hq, hkv, head_dim, rotary, n_q, live, cap):
+    import torch
+    from harness import rel_l2, to_torch_bf16
+    from oracle import kvm_oracle as O
+    from paper_2609_18935_gb300 import kvm
+    ctx = kvm.Context([kvm.LAYER_ATTN], hq, hkv, head_dim, rotary, 1e4, 8, 64, 64, [cap], 8)
+    pos = np.cumsum(np.random.default_rng(3).integers(1, 4, live)).astype(np.int32)
+    ctx.load_prefix(0, live, int(pos[-1]) + 1, pos)
+    K = W.normal_bf16((83, 0), (hkv, live, head_dim))
+    V = W.normal_bf16((83, 1), (hkv, live, head_dim))
+    ctx.set_kv(0, 0, to_torch_bf16(K).cuda(), to_torch_bf16(V).cuda())
+    q = W.normal_bf16((83, 2), (n_q, hq, head_dim))
+    got, _ = ctx.attn_probe(0, 0, to_torch_bf16(q).cuda())
+    ctx.check()
+    ref = O.attention_probe(O.AttnCache(O.bf16_to_f64(K), O.bf16_to_f64(V), pos.astype(np.int64)), O.bf16_to_f64(q),
+                            rotary, 1e4)
+    # fp32 sums: scores of size ~|q||k|/sqrt(D) <= 60 rounded to 2^-24 relative a
+    # few times over, so exp() moves by at most ~60 * 8 * 2^-24
+    assert rel_l2(got.cpu().numpy().astype(np.float64), ref) <= 60 * 8 * 2.0 ** -24
