@@ -181,7 +181,37 @@ __global__ void gather_map_kernel(const __grid_constant__ GatherParams p) {
     }
 }
 
+// grid (x, rows, arrays): 16-byte vectors of one row, four in flight a thread,
+// then its last words.
+__global__ void __launch_bounds__(256) copy_kernel(const __grid_constant__ CopyParams p) {
+    grid_dependency_wait();
+    grid_dependents_launch();
+    const uint8_t* src = p.src[blockIdx.z] + blockIdx.y * p.spitch;
+    uint8_t* dst = p.dst[blockIdx.z] + blockIdx.y * p.dpitch;
+    const uint4* s4 = reinterpret_cast<const uint4*>(src);
+    uint4* d4 = reinterpret_cast<uint4*>(dst);
+    const int64_t n = p.bytes / 16, step = (int64_t)gridDim.x * 256;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += 4 * step) {
+        uint4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * step < n) x[u] = s4[i + u * step];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * step < n) d4[i + u * step] = x[u];
+    }
+    const int64_t w = n * 4 + threadIdx.x;                  // in words
+    if (blockIdx.x == 0 && w < p.bytes / 4)
+        reinterpret_cast<uint32_t*>(dst)[w] = reinterpret_cast<const uint32_t*>(src)[w];
+}
+
 }  // namespace
+
+void launch_copy(const CopyParams& p, cudaStream_t s) {
+    // up to eight blocks an SM, at least four vectors a thread
+    const int64_t per_row = (p.bytes / 16 + 1023) / 1024, most = 8 * (int64_t)p.num_sms / (p.rows * p.n) + 1;
+    launch_pdl(copy_kernel, dim3((unsigned)(per_row < 1 ? 1 : per_row < most ? per_row : most), p.rows, p.n), dim3(256), 0, s, p);
+}
 
 void launch_kv_compact(const CompactParams& p, cudaStream_t s) {
     if (p.total_blocks <= 0) return;

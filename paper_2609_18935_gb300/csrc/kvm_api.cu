@@ -13,6 +13,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <numeric>
 #include <string>
 #include <vector>
 
@@ -75,6 +76,7 @@ struct kvm_ctx {
     // model
     int n_layers = 0;
     std::vector<int> kind, attn_idx, gdn_idx;
+    std::vector<std::string> layer_name;  // of its NVTX range
     int n_attn = 0, n_gdn = 0;
     int Hq = 0, Hkv = 0, D = 0, R = 0, g = 0;
     double theta = 0;
@@ -460,6 +462,7 @@ extern "C" kvm_status kvm_create(const kvm_model_desc* m, int32_t n_chars, const
         const int k = m->layer_kind[l];
         if (k != KVM_LAYER_ATTN && k != KVM_LAYER_GDN) { delete c; return fail(KVM_E_INVAL, "bad layer kind"); }
         c->kind.push_back(k);
+        c->layer_name.push_back("layer " + std::to_string(l) + (k == KVM_LAYER_ATTN ? " (attention)" : " (delta rule)"));
         c->attn_idx.push_back(k == KVM_LAYER_ATTN ? c->n_attn++ : -1);
         c->gdn_idx.push_back(k == KVM_LAYER_GDN ? c->n_gdn++ : -1);
     }
@@ -656,6 +659,54 @@ extern "C" kvm_status kvm_load_prefix(kvm_ctx* c, int32_t b, int32_t live, int64
     return KVM_OK;
 }
 
+namespace {
+// Copies of the state accessors: `rows` pieces of `bytes` bytes each, a row
+// pitch on either side, of up to two arrays.  A kernel of the library follows
+// and precedes its neighbours with the overlapped launches of all the others
+// and costs the host a third of a memcpy call; memory of another device than
+// the current one, or off the 16-byte grid, goes through cudaMemcpy2DAsync.
+kvm_status copy_state(kvm_ctx* c, void* const* dst, const void* const* src, int n, size_t dpitch, size_t spitch,
+                      size_t bytes, int rows, cudaStream_t s) {
+    if (!bytes || !rows) return KVM_OK;
+    int dev = -1;
+    CUDA_TRY(cudaGetDevice(&dev));
+    uintptr_t bits = (uintptr_t)(rows > 1 ? dpitch | spitch : 0);
+    for (int i = 0; i < n; ++i) bits |= reinterpret_cast<uintptr_t>(dst[i]) | reinterpret_cast<uintptr_t>(src[i]);
+    if (dev != c->device || (bits & 15)) {
+        for (int i = 0; i < n; ++i)
+            CUDA_TRY(rows > 1 ? cudaMemcpy2DAsync(dst[i], dpitch, src[i], spitch, bytes, rows, cudaMemcpyDeviceToDevice, s)
+                              : cudaMemcpyAsync(dst[i], src[i], bytes, cudaMemcpyDeviceToDevice, s));
+        return KVM_OK;
+    }
+    CopyParams p;
+    p.n = n;
+    p.rows = rows;
+    for (int i = 0; i < 2; ++i) {
+        p.dst[i] = static_cast<uint8_t*>(i < n ? dst[i] : nullptr);
+        p.src[i] = static_cast<const uint8_t*>(i < n ? src[i] : nullptr);
+    }
+    p.dpitch = (int64_t)dpitch;
+    p.spitch = (int64_t)spitch;
+    p.bytes = (int64_t)bytes;
+    p.num_sms = c->num_sms;
+    ++c->launches;
+    launch_copy(p, s);
+    LAUNCH_CHECK(c);
+    return KVM_OK;
+}
+
+// KV of character b in attention layer `layer`: slab rows of every KV head.
+kvm_status copy_kv(kvm_ctx* c, int layer, int b, void* k, void* v, bool in, cudaStream_t s) {
+    const int L = c->live[b];
+    const size_t row = (size_t)c->D * 2, slab = (size_t)c->T_cap * row;
+    const size_t at = ((size_t)c->attn_idx[layer] * c->Hkv) * slab + (size_t)c->cap_off[b] * row;
+    void* own[2] = {reinterpret_cast<char*>(c->K) + at, reinterpret_cast<char*>(c->V) + at};
+    void* user[2] = {k, v};
+    return in ? copy_state(c, own, user, 2, slab, L * row, L * row, c->Hkv, s)
+              : copy_state(c, user, own, 2, L * row, slab, L * row, c->Hkv, s);
+}
+}  // namespace
+
 extern "C" kvm_status kvm_set_kv(kvm_ctx* c, int32_t layer, int32_t b, const void* k, const void* v,
                                  void* stream) {
     if (!c) return fail(KVM_E_INVAL, "NULL context");
@@ -665,15 +716,7 @@ extern "C" kvm_status kvm_set_kv(kvm_ctx* c, int32_t layer, int32_t b, const voi
     const int L = c->live[b];
     if (L == 0) return KVM_OK;
     if (!k || !v) return fail(KVM_E_INVAL, "NULL k or v");
-    const size_t row = (size_t)c->D * 2;
-    const size_t slab = (size_t)c->T_cap * row;
-    const int a = c->attn_idx[layer];
-    char* kd = reinterpret_cast<char*>(c->K) + ((size_t)a * c->Hkv) * slab + (size_t)c->cap_off[b] * row;
-    char* vd = reinterpret_cast<char*>(c->V) + ((size_t)a * c->Hkv) * slab + (size_t)c->cap_off[b] * row;
-    cudaStream_t s = (cudaStream_t)stream;
-    CUDA_TRY(cudaMemcpy2DAsync(kd, slab, k, L * row, L * row, c->Hkv, cudaMemcpyDeviceToDevice, s));
-    CUDA_TRY(cudaMemcpy2DAsync(vd, slab, v, L * row, L * row, c->Hkv, cudaMemcpyDeviceToDevice, s));
-    return KVM_OK;
+    return copy_kv(c, layer, b, const_cast<void*>(k), const_cast<void*>(v), true, (cudaStream_t)stream);
 }
 
 extern "C" kvm_status kvm_get_kv(kvm_ctx* c, int32_t layer, int32_t b, void* k, void* v, void* stream) {
@@ -684,15 +727,7 @@ extern "C" kvm_status kvm_get_kv(kvm_ctx* c, int32_t layer, int32_t b, void* k, 
     const int L = c->live[b];
     if (L == 0) return KVM_OK;
     if (!k || !v) return fail(KVM_E_INVAL, "NULL k or v");
-    const size_t row = (size_t)c->D * 2;
-    const size_t slab = (size_t)c->T_cap * row;
-    const int a = c->attn_idx[layer];
-    const char* ks = reinterpret_cast<const char*>(c->K) + ((size_t)a * c->Hkv) * slab + (size_t)c->cap_off[b] * row;
-    const char* vs = reinterpret_cast<const char*>(c->V) + ((size_t)a * c->Hkv) * slab + (size_t)c->cap_off[b] * row;
-    cudaStream_t s = (cudaStream_t)stream;
-    CUDA_TRY(cudaMemcpy2DAsync(k, L * row, ks, slab, L * row, c->Hkv, cudaMemcpyDeviceToDevice, s));
-    CUDA_TRY(cudaMemcpy2DAsync(v, L * row, vs, slab, L * row, c->Hkv, cudaMemcpyDeviceToDevice, s));
-    return KVM_OK;
+    return copy_kv(c, layer, b, k, v, false, (cudaStream_t)stream);
 }
 
 extern "C" kvm_status kvm_get_positions(kvm_ctx* c, int32_t b, int32_t* out, void* stream) {
@@ -700,9 +735,9 @@ extern "C" kvm_status kvm_get_positions(kvm_ctx* c, int32_t b, int32_t* out, voi
     if (b < 0 || b >= c->B) return fail(KVM_E_INVAL, "character %d out of range", b);
     if (c->live[b] == 0 || c->n_attn == 0) return KVM_OK;
     if (!out) return fail(KVM_E_INVAL, "NULL output");
-    CUDA_TRY(cudaMemcpyAsync(out, c->pos + c->cap_off[b], (size_t)c->live[b] * 4, cudaMemcpyDeviceToDevice,
-                             (cudaStream_t)stream));
-    return KVM_OK;
+    void* dst = out;
+    const void* src = c->pos + c->cap_off[b];
+    return copy_state(c, &dst, &src, 1, 0, 0, (size_t)c->live[b] * 4, 1, (cudaStream_t)stream);
 }
 
 extern "C" kvm_status kvm_set_state(kvm_ctx* c, int32_t layer, const float* S, void* stream) {
@@ -711,9 +746,9 @@ extern "C" kvm_status kvm_set_state(kvm_ctx* c, int32_t layer, const float* S, v
     if (st) return st;
     if (!S) return fail(KVM_E_INVAL, "NULL state");
     const size_t n = (size_t)c->B * c->H * c->dv * c->dk;
-    CUDA_TRY(cudaMemcpyAsync(c->S + (size_t)c->gdn_idx[layer] * n, S, n * 4, cudaMemcpyDeviceToDevice,
-                             (cudaStream_t)stream));
-    return KVM_OK;
+    void* dst = c->S + (size_t)c->gdn_idx[layer] * n;
+    const void* src = S;
+    return copy_state(c, &dst, &src, 1, 0, 0, n * 4, 1, (cudaStream_t)stream);
 }
 
 extern "C" kvm_status kvm_get_state(kvm_ctx* c, int32_t layer, float* S, void* stream) {
@@ -722,9 +757,9 @@ extern "C" kvm_status kvm_get_state(kvm_ctx* c, int32_t layer, float* S, void* s
     if (st) return st;
     if (!S) return fail(KVM_E_INVAL, "NULL state");
     const size_t n = (size_t)c->B * c->H * c->dv * c->dk;
-    CUDA_TRY(cudaMemcpyAsync(S, c->S + (size_t)c->gdn_idx[layer] * n, n * 4, cudaMemcpyDeviceToDevice,
-                             (cudaStream_t)stream));
-    return KVM_OK;
+    void* dst = S;
+    const void* src = c->S + (size_t)c->gdn_idx[layer] * n;
+    return copy_state(c, &dst, &src, 1, 0, 0, n * 4, 1, (cudaStream_t)stream);
 }
 
 namespace {
@@ -1008,15 +1043,13 @@ void apply_plan(kvm_ctx* c, const SpanPlan& pl, const int32_t* span_cu, const in
     for (int b = 0; b < c->B; ++b) {
         if (pl.n_seg[b] == 0) continue;
         std::vector<int32_t>& P = c->hpos[b];
-        std::vector<int32_t> keep;
-        keep.reserve(pl.L_new[b]);
-        int k = span_cu[b];
-        for (int i = 0; i < (int)P.size(); ++i) {
-            while (k < span_cu[b + 1] && i >= send[k]) ++k;
-            if (k < span_cu[b + 1] && i >= sbeg[k]) continue;
-            keep.push_back(P[i]);
+        int at = sbeg[span_cu[b]];                   // survivors move down span by span, in place
+        for (int k = span_cu[b]; k < span_cu[b + 1]; ++k) {
+            const int from = send[k], to = k + 1 < span_cu[b + 1] ? sbeg[k + 1] : (int)P.size();
+            std::memmove(P.data() + at, P.data() + from, sizeof(int32_t) * (size_t)(to - from));
+            at += to - from;
         }
-        P.swap(keep);
+        P.resize(at);
         c->live[b] = pl.L_new[b];
     }
 }
@@ -1345,7 +1378,10 @@ void do_advance(kvm_ctx* c, const int32_t* tail_cu, const int32_t* tail_pos = nu
             }
             c->cursor[b] = top;
         } else {
-            for (int i = 0; i < m; ++i) c->hpos[b].push_back((int32_t)(c->cursor[b] + i));
+            std::vector<int32_t>& P = c->hpos[b];
+            const size_t n = P.size();
+            P.resize(n + m);
+            std::iota(P.begin() + n, P.end(), (int32_t)c->cursor[b]);
             c->cursor[b] += m;
         }
         c->live[b] += m;
@@ -1541,8 +1577,8 @@ kvm_status update_round_impl(kvm_ctx* c, const kvm_round* r, void* stream) {
     if (st) return st;
     if (!r->q || !r->k || !r->v || !r->out) return fail(KVM_E_INVAL, "NULL per-layer pointer array");
     // validate everything before the first launch: spans and capacity after removal
+    SpanPlan pl;
     {
-        SpanPlan pl;
         st = plan_spans(c, r->span_cu, r->span_begin, r->span_end, pl);
         if (st) return st;
         for (int b = 0; b < c->B; ++b) {
@@ -1631,9 +1667,6 @@ kvm_status update_round_impl(kvm_ctx* c, const kvm_round* r, void* stream) {
     for (int l = c->n_layers - 1; l >= 0; --l)
         if (c->kind[l] == KVM_LAYER_ATTN) first_attn = l;
     const bool side = first_attn > 0 && first_attn < c->n_layers;
-    SpanPlan pl;
-    st = plan_spans(c, r->span_cu, r->span_begin, r->span_end, pl);
-    if (st) return st;
     // piece a runs beside the layers from piece_at[a] up to its attention layer
     std::vector<int> piece_at(c->n_attn, 0);
     for (int l = 0, prev = -1; l < c->n_layers; ++l)
@@ -1710,9 +1743,7 @@ kvm_status update_round_impl(kvm_ctx* c, const kvm_round* r, void* stream) {
             out = c->stage + c->stage_out_off[l];
         }
         {
-            char name[48];
-            snprintf(name, sizeof name, "layer %d (%s)", l, attn ? "attention" : "delta rule");
-            NvtxRange range(name);
+            NvtxRange range(c->layer_name[l].c_str());
             st = attn ? do_attention(c, l, r->tail_cu, q, k, v, out, s, with_pos ? c->tail_pos_dev : nullptr,
                                      with_pos ? r->tail_pos : nullptr)
                       : do_gdn(c, l, r->tail_cu, q, k, v, al, be, out, s);

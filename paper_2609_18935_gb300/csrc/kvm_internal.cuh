@@ -104,6 +104,16 @@ struct GatherParams {
 };
 void launch_gather_map(const GatherParams& p, cudaStream_t s);
 
+// Copies of the state accessors: rows x bytes (a multiple of 4) of up to two
+// arrays, every row 16-byte aligned on both sides.
+struct CopyParams {
+    int32_t n, rows, num_sms;
+    uint8_t* dst[2];
+    const uint8_t* src[2];
+    int64_t dpitch, spitch, bytes;
+};
+void launch_copy(const CopyParams& p, cudaStream_t s);
+
 // ----------------------------------------------------------------------------
 // tail attention
 // ----------------------------------------------------------------------------

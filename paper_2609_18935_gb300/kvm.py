@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 
 import numpy as np
 
@@ -48,6 +49,16 @@ class Round(C.Structure):
                 ("delim_end", C.POINTER(C.c_int32))]
 
 
+class _RoundArgs(C.Structure):
+    """Round, filled from byte strings (index and pointer arrays) instead of
+    typed pointers, which cost more to make than the rest of a small call."""
+    _fields_ = [(name, C.c_char_p if isinstance(kind, type) and issubclass(kind, C._Pointer) else kind)
+                for name, kind in Round._fields_]
+
+
+# Host arrays of the calls on the hot path: bytes, or any ctypes pointer.
+_HOST = C.c_void_p
+
 # name -> (restype, argtypes)
 _SIGS = {
     "kvm_create": (C.c_int, [C.POINTER(ModelDesc), C.c_int32, C.POINTER(C.c_int32), C.c_int32,
@@ -68,20 +79,19 @@ _SIGS = {
     "kvm_spans_from_positions": (C.c_int, [C.c_void_p, C.c_int32, C.c_int32, C.POINTER(C.c_int64),
                                            C.POINTER(C.c_int64), C.POINTER(C.c_int32),
                                            C.POINTER(C.c_int32)]),
-    "kvm_kv_compact": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
-                                 C.POINTER(C.c_int32), C.c_void_p, C.c_void_p]),
-    "kvm_tail_attn_prefill": (C.c_int, [C.c_void_p, C.c_int32, C.POINTER(C.c_int32), C.c_void_p,
+    "kvm_kv_compact": (C.c_int, [C.c_void_p, _HOST, _HOST, _HOST, C.c_void_p, C.c_void_p]),
+    "kvm_tail_attn_prefill": (C.c_int, [C.c_void_p, C.c_int32, _HOST, C.c_void_p,
                                         C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
-    "kvm_gdn_chunk_scan_from_state": (C.c_int, [C.c_void_p, C.c_int32, C.POINTER(C.c_int32), C.c_void_p,
+    "kvm_gdn_chunk_scan_from_state": (C.c_int, [C.c_void_p, C.c_int32, _HOST, C.c_void_p,
                                                 C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                                 C.c_void_p, C.c_void_p]),
-    "kvm_advance": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32)]),
-    "kvm_tail_attn_prefill_at": (C.c_int, [C.c_void_p, C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
+    "kvm_advance": (C.c_int, [C.c_void_p, _HOST]),
+    "kvm_tail_attn_prefill_at": (C.c_int, [C.c_void_p, C.c_int32, _HOST, _HOST,
                                            C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
-    "kvm_advance_at": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
+    "kvm_advance_at": (C.c_int, [C.c_void_p, _HOST, _HOST]),
     "kvm_rerotate_keys": (C.c_int, [C.c_void_p, C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32),
                                     C.c_void_p]),
-    "kvm_update_round": (C.c_int, [C.c_void_p, C.POINTER(Round), C.c_void_p]),
+    "kvm_update_round": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p]),
     "kvm_check": (C.c_int, [C.c_void_p, C.c_void_p]),
     "kvm_launch_count": (C.c_int64, [C.c_void_p]),
     "kvm_fork": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p]),
@@ -95,8 +105,7 @@ _SIGS = {
     "kvm_plan_partition": (C.c_int, [C.c_int32, C.POINTER(C.c_int64), C.c_int32, C.POINTER(C.c_int32),
                                      C.POINTER(C.c_int64)]),
     "kvm_kv_compact_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_int64, C.c_int32,
-                                         C.c_int32, C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
-                                         C.POINTER(C.c_int32), C.c_void_p]),
+                                         C.c_int32, C.c_int32, _HOST, _HOST, C.POINTER(C.c_int32), C.c_void_p]),
     "kvm_kv_compact_noalloc_check": (C.c_int, [C.c_void_p]),
     "kvm_debug_compact_wait": (C.c_int, [C.c_void_p, C.c_int32, C.c_int32]),
     "kvm_debug_poke_canary": (C.c_int, [C.c_void_p]),
@@ -149,6 +158,27 @@ def _p32(a: np.ndarray):
     return a.ctypes.data_as(C.POINTER(C.c_int32))
 
 
+def _b32(a) -> bytes:
+    """The int32 values of a host index array, as the bytes a call reads."""
+    return np.asarray(a, dtype=np.int32).tobytes()
+
+
+def _ptrs(addresses) -> bytes:
+    """A host array of device (or pinned host) addresses, as bytes."""
+    return struct.pack("%dP" % len(addresses), *addresses)
+
+
+_torch_module = None
+
+
+def _torch():
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
 def _dptr(t, dtype=None) -> int:
     """Device address of a contiguous torch CUDA tensor (0 for None)."""
     if t is None:
@@ -163,9 +193,11 @@ def _dptr(t, dtype=None) -> int:
 
 
 def _stream(stream) -> int:
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    torch = _torch()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # without a Stream object around it
+    return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
 
 
 def kv_compact_noalloc(K, V, positions, live, span_begin, span_end, stream=None) -> int:
@@ -186,13 +218,13 @@ def kv_compact_noalloc(K, V, positions, live, span_begin, span_end, stream=None)
             raise ValueError(f"{name} must live on the current CUDA device (cuda:{dev})")
     if positions is not None and positions.numel() < rows:
         raise ValueError(f"positions holds {positions.numel()} entries, need >= slab_rows = {rows}")
-    sb, se = _i32(span_begin), _i32(span_end)
+    sb, se = _b32(span_begin), _b32(span_end)
     if len(sb) != len(se):
         raise ValueError("span_begin and span_end differ in length")
     new_live = C.c_int32()
     _check(_lib.kvm_kv_compact_noalloc(_dptr(K, torch.bfloat16), _dptr(V, torch.bfloat16),
-                                       _dptr(positions, torch.int32), n_slabs, rows, D, int(live), len(sb),
-                                       _p32(sb), _p32(se), C.byref(new_live), _stream(stream)))
+                                       _dptr(positions, torch.int32), n_slabs, rows, D, int(live), len(sb) // 4,
+                                       sb, se, C.byref(new_live), _stream(stream)))
     return new_live.value
 
 
@@ -349,12 +381,12 @@ class Context:
         _check(_lib.kvm_load_prefix(self._h, b, int(live), int(cursor), _p32(pos), _stream(stream)))
 
     def set_kv(self, layer, b, k, v, stream=None):
-        import torch
+        torch = _torch()
         _check(_lib.kvm_set_kv(self._h, layer, b, _dptr(k, torch.bfloat16), _dptr(v, torch.bfloat16),
                                _stream(stream)))
 
     def get_kv(self, layer, b, stream=None):
-        import torch
+        torch = _torch()
         live, _ = self.get_live(b)
         k = torch.empty((self.Hkv, live, self.D), dtype=torch.bfloat16, device="cuda")
         v = torch.empty_like(k)
@@ -362,18 +394,18 @@ class Context:
         return k, v
 
     def get_positions(self, b, stream=None):
-        import torch
+        torch = _torch()
         live, _ = self.get_live(b)
         out = torch.empty(live, dtype=torch.int32, device="cuda")
         _check(_lib.kvm_get_positions(self._h, b, _dptr(out), _stream(stream)))
         return out
 
     def set_state(self, layer, S, stream=None):
-        import torch
+        torch = _torch()
         _check(_lib.kvm_set_state(self._h, layer, _dptr(S, torch.float32), _stream(stream)))
 
     def get_state(self, layer, stream=None):
-        import torch
+        torch = _torch()
         S = torch.empty((self.n_chars, self.H, self.dv, self.dk), dtype=torch.float32, device="cuda")
         _check(_lib.kvm_get_state(self._h, layer, _dptr(S), _stream(stream)))
         return S
@@ -412,23 +444,20 @@ class Context:
 
     # ---------------------------------------------------------------- hot path
     def kv_compact(self, span_cu, span_begin, span_end, gather_out=None, stream=None):
-        import torch
-        cu, sb, se = _i32(span_cu), _i32(span_begin), _i32(span_end)
-        _check(_lib.kvm_kv_compact(self._h, _p32(cu), _p32(sb), _p32(se), _dptr(gather_out, torch.int32),
-                                   _stream(stream)))
+        _check(_lib.kvm_kv_compact(self._h, _b32(span_cu), _b32(span_begin), _b32(span_end),
+                                   _dptr(gather_out, _torch().int32), _stream(stream)))
 
     def tail_attn_prefill(self, layer, tail_cu, q, k_new, v_new, out, tail_pos=None, stream=None):
         """kvm_tail_attn_prefill, or kvm_tail_attn_prefill_at when tail_pos
         (host int32 [sum M], one position id per tail token) is given."""
-        import torch
-        cu = _i32(tail_cu)
-        bf = torch.bfloat16
+        cu = _b32(tail_cu)
+        bf = _torch().bfloat16
         if tail_pos is None:
-            _check(_lib.kvm_tail_attn_prefill(self._h, layer, _p32(cu), _dptr(q, bf), _dptr(k_new, bf),
+            _check(_lib.kvm_tail_attn_prefill(self._h, layer, cu, _dptr(q, bf), _dptr(k_new, bf),
                                               _dptr(v_new, bf), _dptr(out, bf), _stream(stream)))
         else:
-            tp = _i32(tail_pos)
-            _check(_lib.kvm_tail_attn_prefill_at(self._h, layer, _p32(cu), _p32(tp), _dptr(q, bf),
+            tp = _b32(tail_pos)
+            _check(_lib.kvm_tail_attn_prefill_at(self._h, layer, cu, tp, _dptr(q, bf),
                                                  _dptr(k_new, bf), _dptr(v_new, bf), _dptr(out, bf),
                                                  _stream(stream)))
 
@@ -440,20 +469,18 @@ class Context:
                                       _p32(np_) if len(np_) else None, _stream(stream)))
 
     def gdn_chunk_scan_from_state(self, layer, tail_cu, q, k, v, alpha, beta, out, stream=None):
-        import torch
-        cu = _i32(tail_cu)
+        torch = _torch()
         bf, f = torch.bfloat16, torch.float32
-        _check(_lib.kvm_gdn_chunk_scan_from_state(self._h, layer, _p32(cu), _dptr(q, bf), _dptr(k, bf),
+        _check(_lib.kvm_gdn_chunk_scan_from_state(self._h, layer, _b32(tail_cu), _dptr(q, bf), _dptr(k, bf),
                                                   _dptr(v, bf), _dptr(alpha, f), _dptr(beta, f),
                                                   _dptr(out, bf), _stream(stream)))
 
     def advance(self, tail_cu, tail_pos=None):
-        cu = _i32(tail_cu)
+        cu = _b32(tail_cu)
         if tail_pos is None:
-            _check(_lib.kvm_advance(self._h, _p32(cu)))
+            _check(_lib.kvm_advance(self._h, cu))
         else:
-            tp = _i32(tail_pos)
-            _check(_lib.kvm_advance_at(self._h, _p32(cu), _p32(tp)))
+            _check(_lib.kvm_advance_at(self._h, cu, _b32(tail_pos)))
 
     def update_round(self, span_cu, span_begin, span_end, tail_cu, inputs, outputs,
                      io_on_host=False, gather_out=None, stream=None, tail_pos=None, delim=None):
@@ -464,22 +491,20 @@ class Context:
         tail_pos: optional host int32 [sum M] position ids of the tail tokens.
         delim: optional (delim_cu, delim_begin, delim_end), tail-index ranges
         of maintenance delimiters whose KV leave the caches after the round."""
-        n = len(self.layer_kind)
-        arr = lambda: (C.c_void_p * n)()
-        q, k, v, al, be, out = arr(), arr(), arr(), arr(), arr(), arr()
+        q, k, v, al, be, out = [], [], [], [], [], []
         ptr = (lambda t: t.data_ptr() if t is not None else 0)
-        for l in range(n):
+        for l in range(len(self.layer_kind)):
             x = inputs[l]
-            q[l], k[l], v[l] = ptr(x["q"]), ptr(x["k"]), ptr(x["v"])
-            al[l], be[l] = ptr(x.get("alpha")), ptr(x.get("beta"))
-            out[l] = ptr(outputs[l])
-        cu, sb, se, tc = _i32(span_cu), _i32(span_begin), _i32(span_end), _i32(tail_cu)
-        tp = _i32(tail_pos) if tail_pos is not None else None
-        dl = tuple(_i32(x) for x in delim) if delim is not None else None
-        r = Round(_p32(cu), _p32(sb), _p32(se), _p32(tc), q, k, v, al, be, out, int(bool(io_on_host)),
-                  ptr(gather_out), _p32(tp) if tp is not None else None,
-                  *((_p32(dl[0]), _p32(dl[1]), _p32(dl[2])) if dl is not None else (None, None, None)))
-        self._keep = (cu, sb, se, tc, q, k, v, al, be, out, tp, dl)
+            q.append(ptr(x["q"]))
+            k.append(ptr(x["k"]))
+            v.append(ptr(x["v"]))
+            al.append(ptr(x.get("alpha")))
+            be.append(ptr(x.get("beta")))
+            out.append(ptr(outputs[l]))
+        r = _RoundArgs(_b32(span_cu), _b32(span_begin), _b32(span_end), _b32(tail_cu), _ptrs(q), _ptrs(k), _ptrs(v),
+                       _ptrs(al), _ptrs(be), _ptrs(out), int(bool(io_on_host)), ptr(gather_out),
+                       _b32(tail_pos) if tail_pos is not None else None,
+                       *((_b32(x) for x in delim) if delim is not None else (None, None, None)))
         _check(_lib.kvm_update_round(self._h, C.byref(r), _stream(stream)))
 
     def attn_probe(self, layer, b, q, group_of=None, n_groups=0, stream=None):
@@ -487,7 +512,7 @@ class Context:
         entries (CUDA fp32 [live]) for the unrotated queries q (CUDA bf16
         [n_q][Hq][D]) of its last n_q live entries, and the per-group mass
         (CUDA fp32 [n_groups]) when group_of (CUDA int32 [live]) is given."""
-        import torch
+        torch = _torch()
         live, _ = self.get_live(b)
         probs = torch.empty(live, dtype=torch.float32, device="cuda")
         mass = torch.empty(max(1, n_groups), dtype=torch.float32, device="cuda") if group_of is not None else None
