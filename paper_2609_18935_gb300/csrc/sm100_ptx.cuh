@@ -304,6 +304,11 @@ __device__ __forceinline__ void named_bar_sync(int id, int count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
+// Arrive without waiting: the other threads of the barrier named_bar_sync.
+__device__ __forceinline__ void named_bar_arrive(int id, int count) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
 // named_bar_sync that also returns whether `pred` held on every thread.
 __device__ __forceinline__ bool named_bar_and(int id, int count, bool pred) {
     uint32_t r;
@@ -311,11 +316,6 @@ __device__ __forceinline__ bool named_bar_and(int id, int count, bool pred) {
                  "bar.red.and.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
                  : "=r"(r) : "r"(pred ? 1u : 0u), "r"(id), "r"(count) : "memory");
     return r != 0;
-}
-
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
-                 : "memory");
 }
 
 }  // namespace ptx

@@ -12,9 +12,8 @@
 // DRAM reads (2.9 now) and the layer 1340 us (1015 now), a 16896-token prefill
 // 1790 us (1660 now).
 // The rest is cut into contiguous ranges, one per block (stream-K), balanced by a
-// cost model that
-// charges each unit 1 and each segment a block starts 8 more (the host
-// planner bisects for the smallest per-block cost).  A block's range covers whole
+// cost model that charges each unit 1 and each segment a block starts 8 more (the
+// host planner bisects for the smallest per-block cost).  A block's range covers whole
 // query tiles, whose outputs it normalises and stores directly, and at most
 // one partial tile at each end, whose unnormalised accumulator goes to a
 // workspace slot (2c for block c's first range segment, 2c + 1 for its last) for
@@ -26,26 +25,33 @@
 //               three-stage ring (64 keys x D, 128-byte swizzle); separate
 //               warps keep the two rings from waiting on each other;
 //   warp 1      allocates TMEM and issues S_j = Q K_j^T (tcgen05.mma,
-//               M 128, N 64, K D, Q read from TMEM) into two TMEM buffers;
-//   warp 10     issues O += P_j V_j (M 128, N D, K 64) into the TMEM
-//               accumulator.  Two issuers keep the S stream running ahead of
-//               the softmax while the PV stream follows it.  Each issuer warp
-//               runs its loop converged and one elected lane issues: a lone
+//               M 128, N 64, K D, Q read from TMEM) into TMEM, once the softmax
+//               has read S_{j-1} into registers;
+//   warp 10     issues O += P_j V_j (M 128, N D, K 64, P read from TMEM) into
+//               the TMEM accumulator.  Two issuers keep the S stream running
+//               ahead of the softmax while the PV stream follows it.  Each issuer
+//               warp runs its loop converged and one elected lane issues: a lone
 //               lane in a divergent branch issued the same MMAs at ~1.6x the
 //               cycles per instruction;
-//   warps 2-9   softmax: each query row is shared by the two warps that see
-//               its TMEM lane quarter (warp w reads lanes 32 (w mod 4) ..),
-//               one per 32-key half of S_j.  They stage the segment's Q tile
-//               in TMEM (the next segment's as soon as the last S of the
-//               current one has landed), exchange row maxima through shared
-//               memory and a pair barrier, keep an online softmax in base 2
+//   warps 2-9   softmax: two groups of four warps take the key tiles in turn,
+//               a thread a whole row of S_j (warp w reads TMEM lanes
+//               32 (w mod 4) ..).  The groups keep one online softmax in base 2
 //               with lazy rescaling (the reference max moves only when a
 //               score exceeds it by more than 2^8; the O row is then rescaled
-//               in TMEM, each half its half of the columns) and write P_j as
-//               bf16 into one of two shared buffers in the MMA's swizzled
-//               K-major layout, so that the softmax of tile j+1 does not wait
-//               for PV_j.  At the end of a segment each half stores its half
-//               of the O columns.
+//               in TMEM): a row's reference max passes from tile to tile
+//               through shared memory and a barrier between the two warps of
+//               the quarter, and each group sums its own tiles.  P_j goes back
+//               to TMEM as bf16, into one of two buffers beside S.  Both groups
+//               stage the segment's Q tile in TMEM (the next segment's as soon
+//               as the last S of the current one has landed) and store half of
+//               the O columns each at its end.
+// P in TMEM spares shared memory, which the MMAs and the TMA keep busy, 32 KB
+// of traffic a unit (P written, and read again by the MMA); S then has one
+// buffer, which a thread with a whole row empties at once.  With each row split
+// between two warps, two S buffers and P in shared memory (the same barriers a
+// unit, both warps in lockstep) a layer of 1024 tokens at 32K took 370 us against
+// 349, the population's 1036 : 1010, a 16896-token prefill 1651 : 1621.  Long
+// attention runs at the power limit (SM clock 1.7 - 1.9 GHz).
 // Q lives in TMEM rather than shared memory: S_j then reads only K_j from
 // shared memory, and the space goes to a third K and V stage.
 // Every mbarrier wait is bounded in time.  On expiry the block raises an
@@ -68,7 +74,7 @@ constexpr int kThreads = 64 + kSoftmaxThreads + 64;   // + warp 10 (PV issuer), 
 constexpr int kPvWarp = 10;
 constexpr int kVWarp = 11;
 
-constexpr int STAGES = 3;                     // K and V ring depth
+constexpr int STAGES = 3;                     // K and V ring depth (a fourth of either: the same time or more)
 
 enum Bar { K_FULL = 0, K_EMPTY = 3, V_FULL = 6, V_EMPTY = 9, S_FULL = 12, S_EMPTY = 14, P_FULL = 16,
            PV_DONE = 18, Q_FULL = 20, O_FINAL = 21, O_EMPTY = 22, DRAIN_S = 23, DRAIN_PV = 24, N_BARS = 25 };
@@ -78,20 +84,20 @@ struct Cfg {
     static constexpr int NREG = D / 64;                    // 64-column (128-byte) regions
     static constexpr int HALF = D / 2;                     // O columns per softmax half
     static constexpr int KV_BYTES = BN * D * 2;
-    static constexpr int P_BYTES = BM * BN * 2;
     static constexpr int OFF_K = 0;
     static constexpr int OFF_V = OFF_K + STAGES * KV_BYTES;
-    static constexpr int OFF_P = OFF_V + STAGES * KV_BYTES;
-    static constexpr int OFF_BAR = OFF_P + 2 * P_BYTES;
+    static constexpr int OFF_BAR = OFF_V + STAGES * KV_BYTES;
     static constexpr int OFF_SLOT = OFF_BAR + N_BARS * 8;  // TMEM base address
     static constexpr int OFF_ABORT = OFF_SLOT + 4;
-    static constexpr int OFF_X = (OFF_ABORT + 4 + 15) / 16 * 16;   // float [2][2][BM] row exchange
-    static constexpr int USED = OFF_X + 2 * 2 * BM * 4;
+    static constexpr int OFF_X = (OFF_ABORT + 4 + 15) / 16 * 16;   // float [2][2][BM]: (sum, reference max) of each group at a segment's end
+    static constexpr int OFF_MR = OFF_X + 2 * 2 * BM * 4;  // float [BM]: the rows' reference maxima
+    static constexpr int USED = OFF_MR + BM * 4;
     // head_dim 256 leaves no room to align the base up: a block without static
     // shared variables gets a 1024-aligned dynamic base (checked at run time)
     static constexpr int SLACK = (D == 256) ? 0 : 1024;
     static constexpr int SMEM = USED + SLACK;
-    static constexpr uint32_t TMEM_S = 0;                  // two S buffers of BN columns
+    static constexpr uint32_t TMEM_S = 0;                  // S_j, BN columns
+    static constexpr uint32_t TMEM_P = BN;                 // two P buffers of BN / 2 columns: bf16 pairs
     static constexpr uint32_t TMEM_O = 2 * BN;             // D columns
     static constexpr uint32_t TMEM_Q = 2 * BN + D;         // D / 2 columns: Q as bf16 pairs
     static constexpr uint32_t TMEM_COLS = (TMEM_Q + D / 2 <= 256) ? 256 : 512;
@@ -137,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
         return;                                    // uniform: before any barrier or TMEM use
     }
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t sK = sbase + C::OFF_K, sV = sbase + C::OFF_V, sP = sbase + C::OFF_P;
+    const uint32_t sK = sbase + C::OFF_K, sV = sbase + C::OFF_V;
     auto bar = [&](int i) -> uint32_t { return sbase + C::OFF_BAR + 8u * i; };
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_SLOT);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_ABORT);
@@ -175,8 +181,8 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(bar(S_FULL + s), 1);
-            mbar_init(bar(S_EMPTY + s), kSoftmaxThreads);
-            mbar_init(bar(P_FULL + s), kSoftmaxThreads);
+            mbar_init(bar(S_EMPTY + s), kSoftmaxThreads / 2);
+            mbar_init(bar(P_FULL + s), kSoftmaxThreads / 2);
             mbar_init(bar(PV_DONE + s), 1);
         }
         mbar_init(bar(Q_FULL), kSoftmaxThreads);
@@ -251,19 +257,20 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
             const int n = key_end(seg, T.nk) - key_begin(seg);
             ok = warp_wait(bar(Q_FULL), seg & 1, 0x21 + 256 * seg);
             for (int i = 0; i < n && ok; ++i, ++j) {
-                const int sb = j & 1, st = j % STAGES;
+                const int st = j % STAGES;
                 ok = warp_wait(bar(K_FULL + st), (j / STAGES) & 1, 0x22 + 256 * j);
-                if (ok && j >= 2) ok = warp_wait(bar(S_EMPTY + sb), ((j >> 1) - 1) & 1, 0x23 + 256 * j);
+                // S_{j-1} has been read into registers
+                if (ok && j >= 1) ok = warp_wait(bar(S_EMPTY + ((j - 1) & 1)), ((j - 1) >> 1) & 1, 0x23 + 256 * j);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t kd = k_desc0 + (uint64_t)((st * C::KV_BYTES) >> 4);
-                const uint32_t d = tmem + C::TMEM_S + sb * BN;
+                const uint32_t d = tmem + C::TMEM_S;
                 if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks)
                         mma_bf16_ts(d, tmem + C::TMEM_Q + ks * 8, kd + (uint64_t)((((ks >> 2) * (BN * 128)) + (ks & 3) * 32) >> 4),
                                     id_qk, ks > 0);
-                    mma_commit(bar(S_FULL + sb));
+                    mma_commit(bar(S_FULL + (j & 1)));
                     mma_commit(bar(K_EMPTY + st));
                 }
                 __syncwarp();
@@ -278,7 +285,6 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
     } else if (warp == kPvWarp) {
         // ------------------------------------------------------------ PV issuer (same warp discipline)
         const uint32_t id_pv = idesc_bf16_f32(BM, D, true);
-        const uint64_t p_desc0 = smem_desc_sw128(sP, 16, 1024);
         const uint64_t v_desc0 = smem_desc_sw128(sV, BN * 128, 1024);
         bool ok = true;
         int j = 0;
@@ -293,13 +299,13 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
                 if (ok && i == 0 && seg > 0) ok = warp_wait(bar(O_EMPTY), (seg - 1) & 1, 0x26 + 256 * seg);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t pd = p_desc0 + (uint64_t)((pb * C::P_BYTES) >> 4);
+                const uint32_t pt = tmem + C::TMEM_P + pb * (BN / 2);
                 const uint64_t vd = v_desc0 + (uint64_t)((st * C::KV_BYTES) >> 4);
                 if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < BN / 16; ++ks)
-                        mma_bf16(tmem + C::TMEM_O, pd + (uint64_t)((ks * 32) >> 4), vd + (uint64_t)((ks * 16 * 128) >> 4), id_pv,
-                                 (i > 0 || ks > 0) ? 1u : 0u);
+                        mma_bf16_ts(tmem + C::TMEM_O, pt + ks * 8, vd + (uint64_t)((ks * 16 * 128) >> 4), id_pv,
+                                    (i > 0 || ks > 0) ? 1u : 0u);
                     mma_commit(bar(PV_DONE + pb));
                     mma_commit(bar(V_EMPTY + st));
                 }
@@ -317,12 +323,17 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
         __syncwarp();
     } else {
         // ------------------------------------------------------------ softmax + epilogue
-        const int half = (warp - 2) >> 2;                  // key columns 32 half .. +31 of S
+        const int grp = (warp - 2) >> 2;                   // this warp's key tiles: j mod 2 == grp
         const int quarter = warp & 3;                      // TMEM lanes 32 quarter .. +31
         const int r = quarter * 32 + lane;                 // query row of this thread
         const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-        const int pair_bar = 1 + quarter;
         const float sl = p.scale_log2;
+        float* mrs = reinterpret_cast<float*>(smem + C::OFF_MR);
+        // the two warps of a quarter pass the rows' reference max from tile to
+        // tile: one barrier per direction, arrived at by the warp that wrote it
+        auto hand_over = [&](int j) { named_bar_arrive(1 + quarter + 4 * (j & 1), 64); };
+        auto take_over = [&](int j) { named_bar_sync(1 + quarter + 4 * (j & 1), 64); };
+        const int pair_bar = 9 + quarter;
         // waits do not change the control flow (the pair barriers must stay
         // matched); after an abort they return at once and the results are
         // discarded
@@ -346,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
             constexpr int W = D / 4;                       // 32-bit words of this half
             uint4 v[W / 4];
             const uint4* src = reinterpret_cast<const uint4*>(
-                p.q_rot + ((int64_t)(ch.tail_off + tok) * p.Hq + T.kvh * g + (r % g)) * D + half * (D / 2));
+                p.q_rot + ((int64_t)(ch.tail_off + tok) * p.Hq + T.kvh * g + (r % g)) * D + grp * (D / 2));
 #pragma unroll
             for (int e = 0; e < W / 4; ++e) v[e] = tok < ch.M ? src[e] : make_uint4(0, 0, 0, 0);
             const uint32_t* w = reinterpret_cast<const uint32_t*>(v);
@@ -356,13 +367,13 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
                     uint32_t x[32];
 #pragma unroll
                     for (int e = 0; e < 32; ++e) x[e] = w[c0 + e];
-                    tmem_st32(tmem + lane_off + C::TMEM_Q + half * W + c0, x);
+                    tmem_st32(tmem + lane_off + C::TMEM_Q + grp * W + c0, x);
                 }
             } else {
                 uint32_t x[16];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) x[e] = w[e];
-                tmem_st16(tmem + lane_off + C::TMEM_Q + half * W, x);
+                tmem_st16(tmem + lane_off + C::TMEM_Q + grp * W, x);
             }
             tmem_st_wait();
             tc_fence_before();
@@ -380,68 +391,59 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
             const int tok = T.tok0 + r / g;
             const bool row_valid = tok < ch.M;
             const int lim = ch.L_prev + min(tok, ch.M - 1) + 1;    // keys [0, lim) are visible
-            float mr = -INFINITY;                        // reference max, log2 units
-            float l = 0.f;                               // this half's share of the row sum
-            for (int i = 0; i < n; ++i, ++j) {
-                const int sb = j & 1;
-                wait_fast(S_FULL + sb, (j >> 1) & 1, 0x31 + 256 * j);
+            float mr = -INFINITY;                        // reference max at this group's last tile, log2 units
+            float l = 0.f;                               // this group's share of the row sum, relative to it
+            auto scale_to = [&](float from, float to) { return from == to ? 1.f : from == -INFINITY ? 0.f : ex2(from - to); };
+            for (int i = (j & 1) == grp ? 0 : 1; i < n; i += 2) {
+                const int jj = j + i;                    // jj & 1 == grp: barriers and P buffer
+                wait_fast(S_FULL + grp, (jj >> 1) & 1, 0x31 + 256 * jj);
                 tc_fence_after();
-                uint32_t sa[32];
-                tmem_ld32(tmem + lane_off + C::TMEM_S + sb * BN + 32 * half, sa);
+                uint32_t sa[32], sb[32];
+                tmem_ld32(tmem + lane_off + C::TMEM_S, sa);
+                tmem_ld32(tmem + lane_off + C::TMEM_S + 32, sb);
                 tmem_ld_wait();
                 tc_fence_before();
-                mbar_arrive(bar(S_EMPTY + sb));
+                mbar_arrive(bar(S_EMPTY + grp));
                 // the segment's last S has landed, so no MMA reads Q any more
                 if (i + 1 == n && has_next) stage_q(tile_of(seg + 1));
-                const int key0 = (k + i) * BN + 32 * half;
-                float s[32];
+                const int key0 = (k + i) * BN;
+                if (key0 + BN > lim) {
 #pragma unroll
-                for (int c = 0; c < 32; ++c) s[c] = __uint_as_float(sa[c]);
-                if (key0 + 32 > lim) {
-#pragma unroll
-                    for (int c = 0; c < 32; ++c)
-                        if (key0 + c >= lim) s[c] = -INFINITY;
+                    for (int c = 0; c < 32; ++c) {
+                        if (key0 + c >= lim) sa[c] = 0xff800000u;                // -inf
+                        if (key0 + 32 + c >= lim) sb[c] = 0xff800000u;
+                    }
                 }
-                float m16[16];
+                float m8[8];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) m16[c] = fmaxf(s[c], s[c + 16]);
+                for (int c = 0; c < 8; ++c) m8[c] = fmaxf(__uint_as_float(sa[c]), __uint_as_float(sb[c]));
 #pragma unroll
-                for (int w = 8; w >= 1; w >>= 1)
+                for (int c = 8; c < 32; ++c)
+                    m8[c & 7] = fmaxf(m8[c & 7], fmaxf(__uint_as_float(sa[c]), __uint_as_float(sb[c])));
 #pragma unroll
-                    for (int c = 0; c < w; ++c) m16[c] = fmaxf(m16[c], m16[c + w]);
-                const float pm = m16[0];
-                float* xs = xch + sb * 2 * BM;           // [half][row] of this tile
-                xs[half * BM + r] = pm;
-                named_bar_sync(pair_bar, 64);
-                const float mx2 = fmaxf(pm, xs[(1 - half) * BM + r]) * sl;
-                const bool bump = mx2 > mr + 8.0f;       // also true while mr = -inf and a key is visible
-                const float mr_new = bump ? mx2 : mr;
-                float pv[32];
-                float sum = 0.f;
-                if (mr_new == -INFINITY) {
+                for (int w = 4; w >= 1; w >>= 1)
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) pv[c] = 0.f;
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) pv[c] = ex2(fmaf(s[c], sl, -mr_new));
-                    float a16[16];
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) a16[c] = pv[c] + pv[c + 16];
-#pragma unroll
-                    for (int w = 8; w >= 1; w >>= 1)
-#pragma unroll
-                        for (int c = 0; c < w; ++c) a16[c] += a16[c + w];
-                    sum = a16[0];
+                    for (int c = 0; c < w; ++c) m8[c] = fmaxf(m8[c], m8[c + w]);
+                // the reference max after the previous tile (the other group's)
+                if (jj > 0) take_over(jj - 1);
+                const float mp = i > 0 ? mrs[r] : -INFINITY;
+                const float mx2 = m8[0] * sl;
+                const bool bump = mx2 > mp + 8.0f;       // also true while mp = -inf and a key is visible
+                const float mn = bump ? mx2 : mp;
+                mrs[r] = mn;
+                hand_over(jj);
+                // P buffer grp is free once PV_{jj-2} has completed
+                if (jj >= 2) {
+                    wait_fast(PV_DONE + grp, ((jj >> 1) - 1) & 1, 0x32 + 256 * jj);
+                    tc_fence_after();
                 }
-                const float factor = bump ? ((mr == -INFINITY) ? 0.f : ex2(mr - mr_new)) : 1.f;
-                // P buffer sb is free once PV_{j-2} has completed
-                if (j >= 2) wait_fast(PV_DONE + sb, ((j >> 1) - 1) & 1, 0x32 + 256 * j);
                 if (i > 0 && __any_sync(0xffffffffu, bump)) {
-                    // rescale this half of the O row once PV_{j-1} has landed
-                    wait_all(PV_DONE + (sb ^ 1), ((j - 1) >> 1) & 1, 0x33 + 256 * j);
+                    // rescale the O rows once PV_{jj-1} has landed
+                    const float factor = bump ? scale_to(mp, mn) : 1.f;
+                    wait_all(PV_DONE + (grp ^ 1), ((jj - 1) >> 1) & 1, 0x33 + 256 * jj);
                     tc_fence_after();
 #pragma unroll 1
-                    for (int c0 = half * C::HALF; c0 < (half + 1) * C::HALF; c0 += 32) {
+                    for (int c0 = 0; c0 < D; c0 += 32) {
                         uint32_t o[32];
                         tmem_ld32(tmem + lane_off + C::TMEM_O + c0, o);
                         tmem_ld_wait();
@@ -451,32 +453,48 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
                     }
                     tmem_st_wait();
                 }
-                l = l * factor + sum;
-                mr = mr_new;
-                // 32 bf16 of row r = 16-byte chunks 4 half .. 4 half + 3, chunk index XOR (r & 7)
-                const uint32_t prow = sP + sb * C::P_BYTES + r * 128;
+                uint32_t pw[32];                         // the row of P, bf16 pairs
+                const float off = mn == -INFINITY ? 0.f : mn;                    // no visible key yet: every score is -inf
+                float sum4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t w[4];
+                for (int q = 0; q < 8; ++q) {
+                    float pv[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        pv[e] = ex2(fmaf(__uint_as_float(q < 4 ? sa[(8 * q + e) & 31] : sb[(8 * q + e) & 31]), sl, -off));
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        __nv_bfloat162 h2 = __floats2bfloat162_rn(pv[8 * q + 2 * e], pv[8 * q + 2 * e + 1]);
-                        w[e] = *reinterpret_cast<uint32_t*>(&h2);
+                        sum4[e] += pv[2 * e] + pv[2 * e + 1];
+                        __nv_bfloat162 h2 = __floats2bfloat162_rn(pv[2 * e], pv[2 * e + 1]);
+                        pw[4 * q + e] = *reinterpret_cast<uint32_t*>(&h2);
                     }
-                    st_shared_v4(prow + (((4 * half + q) ^ (r & 7)) << 4), w[0], w[1], w[2], w[3]);
                 }
-                fence_proxy_async_smem();
+                tmem_st32(tmem + lane_off + C::TMEM_P + grp * (BN / 2), pw);
+                tmem_st_wait();
                 tc_fence_before();
-                mbar_arrive(bar(P_FULL + sb));
+                mbar_arrive(bar(P_FULL + grp));
+                l = l * scale_to(mr, mn) + ((sum4[0] + sum4[1]) + (sum4[2] + sum4[3]));
+                mr = mn;
             }
+            // the group without the segment's last tile stages its half of the
+            // next Q too (the tile's S buffer is not filled again before that)
+            if (has_next && ((j + n - 1) & 1) != grp) {
+                wait_all(S_FULL + (grp ^ 1), ((j + n - 1) >> 1) & 1, 0x35 + 256 * j);
+                tc_fence_after();
+                stage_q(tile_of(seg + 1));
+            }
+            j += n;
             // ---------------------------------------------------------------- epilogue of the segment
             wait_all(O_FINAL, seg & 1, 0x34 + 256 * seg);
             tc_fence_after();
-            float* xl = xch + (j & 1) * 2 * BM;          // the exchange buffer the last tile did not use
-            xl[half * BM + r] = l;
+            float* xl = xch;                             // [group][row] sums, then reference maxima
+            xl[grp * BM + r] = l;
+            xl[(2 + grp) * BM + r] = mr;
             named_bar_sync(pair_bar, 64);
-            const float lt = l + xl[(1 - half) * BM + r];
+            const float lo = xl[(1 - grp) * BM + r], mo = xl[(3 - grp) * BM + r];
             named_bar_sync(pair_bar, 64);                // the buffer is free for the next segment
+            const float mfin = fmaxf(mr, mo);
+            const float lt = l * scale_to(mr, mfin) + lo * scale_to(mo, mfin);
             const bool store = *abort_flag == 0;
             const int hq = T.kvh * g + (r % g);
             if (full) {
@@ -484,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
                 const float inv = row_valid ? 1.f / lt : 0.f;
                 __nv_bfloat16* o = p.out + ((int64_t)(ch.tail_off + (row_valid ? tok : 0)) * p.Hq + hq) * D;
 #pragma unroll 1
-                for (int c0 = half * C::HALF; c0 < (half + 1) * C::HALF; c0 += 32) {
+                for (int c0 = grp * C::HALF; c0 < (grp + 1) * C::HALF; c0 += 32) {
                     uint32_t v[32];
                     tmem_ld32(tmem + lane_off + C::TMEM_O + c0, v);
                     tmem_ld_wait();
@@ -504,15 +522,15 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
                 }
             } else {
                 const int64_t prow = (int64_t)(2 * cta + (seg == waves ? 0 : 1)) * BM + r;
-                if (half == 0 && store && row_valid) {       // only real rows are merged
-                    p.part_ml[prow * 2 + 0] = mr;
+                if (grp == 0 && store && row_valid) {       // only real rows are merged
+                    p.part_ml[prow * 2 + 0] = mfin;
                     p.part_ml[prow * 2 + 1] = lt;
                 }
                 // partial layout [slot][D / 32][8][row][4]: each 16-byte store
                 // of a warp lands in 512 contiguous bytes
                 const int64_t slot = 2 * cta + (seg == waves ? 0 : 1);
 #pragma unroll 1
-                for (int c0 = half * C::HALF; c0 < (half + 1) * C::HALF; c0 += 32) {
+                for (int c0 = grp * C::HALF; c0 < (grp + 1) * C::HALF; c0 += 32) {
                     uint32_t v[32];
                     tmem_ld32(tmem + lane_off + C::TMEM_O + c0, v);
                     tmem_ld_wait();
@@ -527,6 +545,7 @@ __global__ void __launch_bounds__(kThreads, 1) tail_attention_tc_kernel(const __
             tc_fence_before();
             mbar_arrive(bar(O_EMPTY));
         }
+        if (j > 0 && (j & 1) == grp) take_over(j - 1);     // the last hand-over finds its partner
     }
     tc_fence_before();
     __syncthreads();
