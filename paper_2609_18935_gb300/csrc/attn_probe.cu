@@ -21,7 +21,7 @@
 // The scores are formed once and pass through memory (the attention's partials
 // workspace; row blocks that do not fit together are done in turn).  8192 keys,
 // 8 queries of 16 heads of 256 (0.54 GFLOP): rotate 4, scores 22,
-// rows 5, probs 13 us alone, 61 together, against 210 with the scores formed
+// rows 5, probs 7 us alone, 56 together, against 210 with the scores formed
 // twice by 128 threads a tile and one thread a row merging the tiles
 // Fp32 products throughout: on the tensor cores the queries would have to be
 // split, and this is the reference that other paths are judged by.
@@ -224,17 +224,30 @@ __global__ void __launch_bounds__(kProbThreads) probe_probs_kernel(const __grid_
     }
     part[w][lane] = acc;
     __syncthreads();
-    if (w > 0 || j >= p.L) return;
+    if (w > 0) return;
     float tot = 0.f;
+    if (j < p.L) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) tot += part[k][lane];
-    if (p.row_block0 > 0) tot += p.probs[j];
-    if (p.last) tot /= (float)(p.n_q * p.Hq);
-    p.probs[j] = tot;
+        for (int k = 0; k < 8; ++k) tot += part[k][lane];
+        if (p.row_block0 > 0) tot += p.probs[j];
+        if (p.last) tot /= (float)(p.n_q * p.Hq);
+        p.probs[j] = tot;
+    }
     if (p.last && p.group_of) {
-        const int gid = p.group_of[j];
+        const int gid = j < p.L ? p.group_of[j] : -1;
         if (gid >= p.n_groups) atomicOr(p.err, kErrBounds);
-        else if (gid >= 0) atomicAdd(p.group_mass + gid, tot);
+        const bool in = gid >= 0 && gid < p.n_groups;
+        // a record's entries are neighbours: one addition a group and warp
+        uint32_t left = __ballot_sync(0xffffffffu, in);
+        while (left) {
+            const int lead = __shfl_sync(0xffffffffu, gid, __ffs(left) - 1);
+            const bool mine = in && gid == lead;
+            float sum = mine ? tot : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == __ffs(left) - 1) atomicAdd(p.group_mass + lead, sum);
+            left &= ~__ballot_sync(0xffffffffu, mine);
+        }
     }
 }
 
