@@ -1819,8 +1819,9 @@ __device__ __forceinline__ void gdn_scan_packed_run(const GdnParams& p, const Fu
 
 template <int DK, int CW>
 __global__ void __launch_bounds__(kThreads, 1) gdn_scan_kernel(const __grid_constant__ GdnParams p) {
-    if constexpr (CW == 16) gdn_scan_packed_run<DK>(p, FuseCtl{nullptr, 0}, blockIdx.z, blockIdx.y, blockIdx.x * p.dv_slice);
-    else gdn_scan_run<DK, CW>(p, FuseCtl{nullptr, 0}, blockIdx.z, blockIdx.y, blockIdx.x * p.dv_slice);
+    const int b = p.order[blockIdx.z];
+    if constexpr (CW == 16) gdn_scan_packed_run<DK>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
+    else gdn_scan_run<DK, CW>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
 }
 
 // ============================================================================

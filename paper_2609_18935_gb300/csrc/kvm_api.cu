@@ -1300,6 +1300,8 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         chunks += (p.ch[b].M + 63) / 64;
     }
     p.total_chunks = chunks;
+    for (int b = 0; b < c->B; ++b) p.order[b] = (int16_t)b;
+    std::stable_sort(p.order, p.order + c->B, [&](int a, int b) { return p.ch[a].M > p.ch[b].M; });
     // two prep blocks per (chunk, head) when both fit on the SMs at once: they
     // share the solve for X and halve the products, staging and record
     // stores that follow it

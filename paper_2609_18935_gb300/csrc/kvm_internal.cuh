@@ -274,6 +274,9 @@ struct GdnParams {
     uint8_t* snap;
     int64_t snap_bytes;
     GdnChar ch[kMaxChars];
+    // characters by decreasing tail: a population's longest chains start first
+    // (32 characters of 64 .. 512 tokens, 16 heads: 107 -> 94 us)
+    int16_t order[kMaxChars];
 };
 
 // Short convolution (width 4) + SiLU of a delta-rule layer's q/k/v with the
