@@ -35,15 +35,20 @@ __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Old (source) index of new index j >= first, for one character.
-__device__ __forceinline__ int src_index(const int32_t* seg_start, const int32_t* seg_shift,
-                                         int n_seg, int j) {
-    int lo = 0, hi = n_seg - 1;            // last k with seg_start[k] <= j
+// Segment of new index j >= first, for one character: the last one that starts
+// at or before it.
+__device__ __forceinline__ int seg_of(const int32_t* seg_start, int n_seg, int j) {
+    int lo = 0, hi = n_seg - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
         if (seg_start[mid] <= j) lo = mid; else hi = mid - 1;
     }
-    return j + seg_shift[lo];
+    return lo;
+}
+// Old (source) index of new index j >= first.
+__device__ __forceinline__ int src_index(const int32_t* seg_start, const int32_t* seg_shift,
+                                         int n_seg, int j) {
+    return j + seg_shift[seg_of(seg_start, n_seg, j)];
 }
 
 __global__ void __launch_bounds__(kCompactThreads)
@@ -61,7 +66,10 @@ kv_compact_kernel(const __grid_constant__ CompactParams p) {
     const CompactChar& c = p.ch[b];
     const int local = blockIdx.x - c.blk_off;
     const bool is_pos = local >= p.n_kv_slabs * c.chunks_kv;
-    const int slab = is_pos ? p.n_kv_slabs : local / c.chunks_kv;
+    // neighbouring blocks take chunks of different slabs: a chunk's neighbours in
+    // its own slab, whose sources it overwrites, were read long before (slab after
+    // slab, 1.5 GB in 48 slabs took 327 us, now 260, 5.7 TB/s)
+    const int slab = is_pos ? p.n_kv_slabs : local % p.n_kv_slabs;
     const int n_chunks = is_pos ? c.chunks_pos : c.chunks_kv;
     const int rows = is_pos ? p.rows_pos : p.rows_kv;
     const int32_t* seg_start = p.seg_start + c.seg_off;
@@ -93,13 +101,24 @@ kv_compact_kernel(const __grid_constant__ CompactParams p) {
         const int s_in = slab < half ? slab : slab - half;
         base = arr + ((int64_t)s_in * p.slab_rows + c.cap_off) * p.vec_per_row;
         const int n_vec = (d1 - d0) * p.vec_per_row;
+        const int seg0 = seg_of(seg_start, c.n_seg, d0);
+        if (seg0 + 1 == c.n_seg || seg_start[seg0 + 1] >= d1) {
+            // all rows come from one segment: a contiguous piece
+            const uint4* src = base + (int64_t)(d0 + seg_shift[seg0]) * p.vec_per_row;
 #pragma unroll
-        for (int k = 0; k < kCompactVecPerThread; ++k) {
-            const int v = tid + k * kCompactThreads;
-            if (v < n_vec) {
-                const int row = d0 + v / p.vec_per_row;
-                const int src = src_index(seg_start, seg_shift, c.n_seg, row);
-                vbuf[k] = __ldcg(base + (int64_t)src * p.vec_per_row + v % p.vec_per_row);
+            for (int k = 0; k < kCompactVecPerThread; ++k) {
+                const int v = tid + k * kCompactThreads;
+                if (v < n_vec) vbuf[k] = __ldcg(src + v);
+            }
+        } else {
+            const int lg = __ffs(p.vec_per_row) - 1;         // 8, 16 or 32 vectors a row
+#pragma unroll
+            for (int k = 0; k < kCompactVecPerThread; ++k) {
+                const int v = tid + k * kCompactThreads;
+                if (v < n_vec) {
+                    const int src = src_index(seg_start, seg_shift, c.n_seg, d0 + (v >> lg));
+                    vbuf[k] = __ldcg(base + (int64_t)src * p.vec_per_row + (v & (p.vec_per_row - 1)));
+                }
             }
         }
     } else {
@@ -112,21 +131,27 @@ kv_compact_kernel(const __grid_constant__ CompactParams p) {
             }
         }
     }
+    // earlier chunks whose sources reach into [d0, d1) are the last `deps` ones
+    // (their last sources are ordered); warp 0 counts them a chunk a lane while
+    // the loads are in flight
+    int deps = 0;
+    if (tid < 32) {
+        for (int e0 = chunk - 1; e0 >= 0; e0 -= 32) {
+            const int e = e0 - tid;
+            const bool reach = e >= 0 && src_index(seg_start, seg_shift, c.n_seg, min(c.first + (e + 1) * rows, c.L_new) - 1) >= d0;
+            const uint32_t m = __ballot_sync(0xffffffffu, reach);
+            deps += __popc(m);
+            if (m != 0xffffffffu) break;
+        }
+    }
     __threadfence();
     __syncthreads();
     if (tid == 0) st_release(p.flags + (int64_t)(flag_base + chunk) * p.flag_stride, p.epoch);
     if (tid < 32) {
-        // earlier chunks whose sources reach into [d0, d1) are e_min .. chunk - 1
-        // (their last sources are ordered); the lanes of warp 0 wait on their
-        // flags together, one flag each, so the waits cost one round trip
-        int e_min = chunk;
-        for (int e = chunk - 1; e >= 0; --e) {
-            const int last_dst = min(c.first + (e + 1) * rows, c.L_new) - 1;
-            if (src_index(seg_start, seg_shift, c.n_seg, last_dst) < d0) break;
-            e_min = e;
-        }
+        // the lanes of warp 0 wait on their flags together, one flag each, so
+        // the waits cost one round trip
         bool fail = false;
-        for (int e = e_min + tid; e < chunk && !fail; e += 32) {
+        for (int e = chunk - deps + tid; e < chunk && !fail; e += 32) {
             int it = 0;
             while (ld_acquire(p.flags + (int64_t)(flag_base + e) * p.flag_stride) != p.epoch) {
                 if (++it > p.wait_limit) { fail = true; break; }
