@@ -20,8 +20,8 @@
 //
 // The scores are formed once and pass through memory (the attention's partials
 // workspace; row blocks that do not fit together are done in turn).  8192 keys,
-// 8 queries of 16 heads of 256 (0.54 GFLOP): rotate 4, scores 22,
-// rows 5, probs 7 us alone, 56 together, against 210 with the scores formed
+// 8 queries of 16 heads of 256 (0.54 GFLOP): rotate 4, scores 18,
+// rows 5, probs 5 us alone, 48 together, against 210 with the scores formed
 // twice by 128 threads a tile and one thread a row merging the tiles
 // Fp32 products throughout: on the tensor cores the queries would have to be
 // split, and this is the reference that other paths are judged by.
@@ -90,7 +90,9 @@ __global__ void __launch_bounds__(kScoreThreads) probe_scores_kernel(const __gri
     grid_dependency_wait();
     grid_dependents_launch();
     const __nv_bfloat16* kb = p.K + ((int64_t)kv * p.slab_rows + p.slot0 + j0) * D;
-    // staging: thread t moves dims 8 (t mod 4) .. + 7 of tile rows t / 4, t / 4 + 32
+    // staging: thread t moves dims 8 (t mod 4) .. + 7 of tile rows t / 4, t / 4 + 32,
+    // turned by 8 (t mod 4) columns so that the four pieces of a row meet
+    // different banks
     const int c = (tid & 3) * 8, sr = tid >> 2;
     const float* qr[2];
     bool q_in[2], k_in[2];
@@ -126,19 +128,20 @@ __global__ void __launch_bounds__(kScoreThreads) probe_scores_kernel(const __gri
             const float* f = reinterpret_cast<const float*>(&qx[i][0]);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                Ks[c + 2 * e][sr + 32 * i] = __uint_as_float(w[e] << 16);
-                Ks[c + 2 * e + 1][sr + 32 * i] = __uint_as_float(w[e] & 0xffff0000u);
+                Ks[c + 2 * e][(sr + 32 * i + c) & 63] = __uint_as_float(w[e] << 16);
+                Ks[c + 2 * e + 1][(sr + 32 * i + c) & 63] = __uint_as_float(w[e] & 0xffff0000u);
             }
 #pragma unroll
-            for (int e = 0; e < 8; ++e) Qs[c + e][sr + 32 * i] = f[e];
+            for (int e = 0; e < 8; ++e) Qs[c + e][(sr + 32 * i + c) & 63] = f[e];
         }
         __syncthreads();
         if (d0 + kDims < D) load(d0 + kDims);                 // in flight during the products
 #pragma unroll 8
         for (int d = 0; d < kDims; ++d) {
-            const float4 k4 = *reinterpret_cast<const float4*>(&Ks[d][4 * tx]);
-            const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&Qs[d][8 * ty]);
-            const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(&Qs[d][8 * ty + 4]);
+            const int turn = d & ~7;                          // dims 8 k .. 8 k + 7 are stored turned by 8 k columns
+            const float4 k4 = *reinterpret_cast<const float4*>(&Ks[d][(4 * tx + turn) & 63]);
+            const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&Qs[d][(8 * ty + turn) & 63]);
+            const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(&Qs[d][(8 * ty + 4 + turn) & 63]);
             const f2 kk[4] = {pack2(k4.x, k4.x), pack2(k4.y, k4.y), pack2(k4.z, k4.z), pack2(k4.w, k4.w)};
             const f2 qq[4] = {qa.x, qa.y, qb.x, qb.y};
 #pragma unroll
