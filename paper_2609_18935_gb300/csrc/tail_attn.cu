@@ -305,15 +305,15 @@ __global__ void __launch_bounds__(kCombineThreads) attn_combine_group_kernel(con
 
 // Few rows, many parts (decode steps): a query tile of a single token has g
 // rows, and one character's tiles are split over tens of blocks.  A warp of
-// the block takes every 16th part for 32 (row, 4-column piece) items, rows
-// fastest; the 16 results meet in shared memory.  grid (n_split_tiles,
+// the block takes every LANES-th part for 32 (row, 4-column piece) items, rows
+// fastest; the LANES results meet in shared memory.  grid (n_split_tiles,
 // ceil(largest tile's rows * D / 4 / 32)).
-constexpr int kPartLanes = 16;
-__global__ void __launch_bounds__(32 * kPartLanes) attn_combine_parts_kernel(const __grid_constant__ CombineParams p) {
+template <int LANES>
+__global__ void __launch_bounds__(32 * LANES) attn_combine_parts_kernel(const __grid_constant__ CombineParams p) {
     grid_dependency_wait();
     grid_dependents_launch();
-    __shared__ float4 acc_s[kPartLanes][32];
-    __shared__ float2 md_s[kPartLanes][32];
+    __shared__ float4 acc_s[LANES][32];
+    __shared__ float2 md_s[LANES][32];
     const SplitTile st = p.tile[blockIdx.x];
     const int D = p.D, rows = st.rows;
     const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(32 * kPartLanes) attn_combine_parts_kernel(con
         mx = nmx;
     };
 #pragma unroll 2
-    for (int q = part; q < st.n_parts; q += kPartLanes) {
+    for (int q = part; q < st.n_parts; q += LANES) {
         const int slot = part_slot(st, q);
         const float2 ml = *reinterpret_cast<const float2*>(pm + slot * (2 * kRows));
         const float4 x = *reinterpret_cast<const float4*>(po + (int64_t)slot * sstride);
@@ -348,11 +348,11 @@ __global__ void __launch_bounds__(32 * kPartLanes) attn_combine_parts_kernel(con
     if (part > 0 || !act) return;
     float top = -INFINITY;
 #pragma unroll
-    for (int q = 0; q < kPartLanes; ++q) top = fmaxf(top, md_s[q][lane].x);
+    for (int q = 0; q < LANES; ++q) top = fmaxf(top, md_s[q][lane].x);
     den = 0.f;
     acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int q = 0; q < kPartLanes; ++q) {
+    for (int q = 0; q < LANES; ++q) {
         const float2 md = md_s[q][lane];
         const float4 x = acc_s[q][lane];
         const float w = md.x == -INFINITY ? 0.f : exp2f(md.x - top);
@@ -422,12 +422,19 @@ void launch_attn_combine(const CombineParams& p, cudaStream_t s) {
     // few real rows in a tile (decode steps): parts side by side, while that
     // grid is two waves (four blocks an SM).  One character's step at 8K (two
     // tiles, 32 parts each) 4.0 us against 13 in the piece form; with all 128
-    // rows real and two parts (a 64-token tail at head_dim 64) 3.6 against 2.8
-    int rows = 0;
-    for (int x = 0; x < p.n_split_tiles; ++x) rows = max(rows, (int)p.tile[x].rows);
+    // rows real and two parts (a 64-token tail at head_dim 64) 3.6 against 2.8.
+    // Four warps where no tile has more than eight parts: 32 characters' step
+    // (59 tiles of 2 - 4 parts) 8.8 -> 4.6 us
+    int rows = 0, parts = 0;
+    for (int x = 0; x < p.n_split_tiles; ++x) {
+        rows = max(rows, (int)p.tile[x].rows);
+        parts = max(parts, (int)p.tile[x].n_parts);
+    }
     const int part_blocks = (rows * (p.D / 4) + 31) / 32;
     if (rows <= 32 && (int64_t)p.n_split_tiles * part_blocks <= 8 * (int64_t)sms) {
-        launch_pdl(attn_combine_parts_kernel, dim3(p.n_split_tiles, part_blocks), dim3(32 * kPartLanes), 0, s, p);
+        const dim3 grid(p.n_split_tiles, part_blocks);
+        if (parts <= 8) launch_pdl(attn_combine_parts_kernel<4>, grid, dim3(32 * 4), 0, s, p);
+        else launch_pdl(attn_combine_parts_kernel<16>, grid, dim3(32 * 16), 0, s, p);
         return;
     }
     const int piece_blocks = (kRows * (p.D / 4) + 255) / 256;
