@@ -1280,13 +1280,13 @@ struct ScanCfg {
     static constexpr uint32_t T_S = 128;                     // S^T (dv cols)
 };
 
-// CW: columns of the slice a thread handles per TMEM access (16 when the
-// slice is 32 wide, so that all eight warps share the elementwise phases)
-// One scan item: character b, head h, d_v rows r0 .. r0 + dv_slice - 1.
-// Written for 256 threads (eight warps: lane quarter x column half); in a
-// fused launch's 512-thread blocks the other eight warps only take part in
-// the block barriers (their column range is empty).
-template <int DK, int CW>
+// One scan item: character b, head h, d_v rows r0 .. r0 + dv_slice - 1, for
+// slices of more than 32 rows (populations whose items cover the SMs).  128 NH
+// threads: thread (row, column group) handles pieces of CW columns.  NH 4
+// against NH 2 with CW 32: 16 characters of 64 tokens 37.4 -> 35.8 us a layer, 32
+// 79.5 -> 77.7; the rest is the MMAs and the records' way from DRAM, 144 KB a
+// chunk and head.
+template <int DK, int CW, int NH>
 __device__ __forceinline__ void gdn_scan_run(const GdnParams& p, const FuseCtl& fc, int b, int h, int r0) {
     using G = ScanCfg<DK>;
     using R = Rec<DK>;
@@ -1316,7 +1316,7 @@ __device__ __forceinline__ void gdn_scan_run(const GdnParams& p, const FuseCtl& 
     const uint32_t ubytes = 128u * dvs * 4u;         // the block's slice of U | A U
     const int64_t uslice = R::uau_off() + (int64_t)r0 * 128 * 4;
     float* Sg = p.S + ((int64_t)b * H + h) * dv * DK;
-    const int dhalf = ((dvs / 2) + CW - 1) / CW * CW;
+    const int dhalf = ((dvs / NH) + CW - 1) / CW * CW;
     const int dlo = hf * dhalf, dhi = min(dvs, dlo + dhalf);
     auto rec_of = [&](int i) -> const uint8_t* { return p.work + ((int64_t)(ch.chunk_off + i) * H + h) * p.rec_bytes; };
 
@@ -1817,11 +1817,12 @@ __device__ __forceinline__ void gdn_scan_packed_run(const GdnParams& p, const Fu
     }
 }
 
-template <int DK, int CW>
-__global__ void __launch_bounds__(kThreads, 1) gdn_scan_kernel(const __grid_constant__ GdnParams p) {
+// WIDE: slices of more than 32 rows, on 512 threads
+template <int DK, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 512 : kThreads, 1) gdn_scan_kernel(const __grid_constant__ GdnParams p) {
     const int b = p.order[blockIdx.z];
-    if constexpr (CW == 16) gdn_scan_packed_run<DK>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
-    else gdn_scan_run<DK, CW>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
+    if constexpr (WIDE) gdn_scan_run<DK, 16, 4>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
+    else gdn_scan_packed_run<DK>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
 }
 
 // ============================================================================
@@ -2234,17 +2235,17 @@ void launch_prep_dk(const GdnParams& p, cudaStream_t s) {
     }
 }
 
-template <int DK, int CW>
-void launch_scan_cw(const GdnParams& p, cudaStream_t s) {
-    configure_once<gdn_scan_kernel<DK, CW>>(ScanCfg<DK>::SMEM);
+template <int DK, bool WIDE>
+void launch_scan_w(const GdnParams& p, cudaStream_t s) {
+    configure_once<gdn_scan_kernel<DK, WIDE>>(ScanCfg<DK>::SMEM);
     dim3 grid(p.dv / p.dv_slice, p.H, p.n_chars);
-    launch_pdl(gdn_scan_kernel<DK, CW>, grid, dim3(kThreads), ScanCfg<DK>::SMEM, s, p);
+    launch_pdl(gdn_scan_kernel<DK, WIDE>, grid, dim3(WIDE ? 512 : kThreads), ScanCfg<DK>::SMEM, s, p);
 }
 
 template <int DK>
 void launch_scan_dk(const GdnParams& p, cudaStream_t s) {
-    if (p.dv_slice <= 32) launch_scan_cw<DK, 16>(p, s);
-    else launch_scan_cw<DK, 32>(p, s);
+    if (p.dv_slice <= 32) launch_scan_w<DK, false>(p, s);
+    else launch_scan_w<DK, true>(p, s);
 }
 
 template <int DK>
