@@ -78,3 +78,21 @@ def test_an_alpha_of_zero_clears_the_state():
                                   torch.from_numpy(beta).cuda(), out)
     want = 0.75 * O.bf16_to_f64(v)[0][:, :, None] * O.bf16_to_f64(k)[0][:, None, :]
     np.testing.assert_allclose(ctx.get_state(0)[0].cpu().numpy(), want, rtol=2.0 ** -22, atol=0)
+
+
+@pytest.mark.parametrize("heads,dk,dv", [(4, 64, 96), (3, 128, 128)])
+def test_short_tails_after_the_convolution(heads, dk, dv):
+    """The convolution inside the step (a few tokens), in a launch before it, and
+    before the chunked form, with the carried state passed between them: rounds of
+    one population whose tails cross those limits, and empty tails."""
+    from harness import Pair
+    shape = W.ModelShape([W.GDN, W.GDN], 8, 2, 64, 64, 1e4, heads, dk, dv)
+    prefix = [0, 0, 0]
+    pair = Pair(shape, prefix, [256] * 3, 160, seed_index=94, conv=True)
+    w = W.Workload("recur-conv", 94, shape, prefix, 7)
+    for r, tails in enumerate([[1, 2, 0], [4, 3, 1], [0, 0, 2], [5, 9, 32], [33, 1, 0], [1, 1, 1], [48, 49, 2]]):
+        w.plan = [[(0.0, 0, m) for m in tails]] * 7
+        errs = pair.run_round(np.zeros(4, np.int32), np.zeros(0, np.int32), np.zeros(0, np.int32), tails,
+                              W.tail_inputs(w, r, tails))
+        bad = {k: v for k, v in errs.items() if not v <= 5e-3}       # the library's bar, bf16 inputs
+        assert not bad, (r, bad)
