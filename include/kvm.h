@@ -200,7 +200,7 @@ kvm_status kvm_plan_spans_from_positions(int32_t live, const int32_t* positions,
  * merged by the combine kernel).  kvm_tail_attn_prefill uses max_blocks =
  * min(320, the device's SM count); with more than a wave and a half of query
  * tiles it first deals whole tiles to the blocks in waves and cuts only the
- * rest in this way.  Errors: KVM_E_INVAL, KVM_E_UNSUPPORTED. */
+ * rest in this way, and tiles of at most 5 key tiles get a block each.  Errors: KVM_E_INVAL, KVM_E_UNSUPPORTED. */
 kvm_status kvm_plan_attention(int32_t n_chars, const int32_t* live, const int32_t* tail_cu,
                               int32_t n_q_heads, int32_t n_kv_heads, int32_t max_blocks,
                               int32_t* n_blocks, int32_t* n_tiles, int32_t* block_tile,

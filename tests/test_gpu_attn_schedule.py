@@ -26,6 +26,7 @@ CASES = {
     "waves": (32, 4, 64, [150 + 7 * b for b in range(40)], [0 if b == 3 else 128 - b for b in range(40)]),
     "waves_d256": (16, 2, 256, [64 + 11 * b for b in range(24)], [97 + b for b in range(24)]),
     "uneven": (32, 4, 64, [12000] + [5] * 39, [128] * 40),
+    "short": (16, 2, 256, [0, 70, 300], [16, 1, 20]),          # at most five key tiles: a block a tile
     "decode_one": (16, 2, 256, [6000], [1]),
     "decode_many": (16, 4, 128, [900 + 131 * b for b in range(9)], [1, 2, 0, 1, 1, 3, 1, 1, 1]),
 }
