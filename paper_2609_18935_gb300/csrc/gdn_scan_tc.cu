@@ -1831,7 +1831,7 @@ __global__ void __launch_bounds__(WIDE ? 512 : kThreads, 1) gdn_scan_kernel(cons
 // the (chunk, head) units in fused_unit order and publish each record through
 // its flag.  A scan waits only for records, and prep workers never wait, so
 // the launch completes as long as every prep worker eventually gets an SM:
-// the scan items leave two thirds of the SMs, other kernels' blocks
+// the scan items leave half of the SMs, other kernels' blocks
 // (the compaction beside it) finish on their own, and the kernels after it
 // on the stream cannot take an SM before every block of it has started
 // (their launch waits for every block's launch_dependents).  Not a

@@ -1323,17 +1323,17 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     // stores that follow it
     p.num_sms = c->num_sms;
     p.prep_parts = (int64_t)2 * chunks * c->H <= c->num_sms ? 2 : 1;
-    // One launch for both when the scan items leave most SMs to prep workers
+    // One launch for both when the scan items leave half the SMs to prep workers
     // (few characters) and the prep is more than one wave of two blocks an SM
     // (long tails): the chunk scan then starts on the first records while the
     // prep still works on later chunks.  Fused against two launches, us a layer:
-    // 104 workers (12 heads of 128) 89 : 94 at 2048 tokens, 169 : 181 at 4096;
-    // 120 workers (d_k 64) 77 : 88, 154 : 166; but 88 workers (16 heads of 128)
-    // 53 : 51 at 1024 and 203 : 198 at 4096, 24 workers (32 heads) 309 : 76 at
-    // 1024.  Otherwise the prep grid, then the scan.
+    // 88 workers (16 heads of 128) 61 : 69 at 1280 tokens, 95 : 103 at 2048, 190 : 192
+    // at 4096, the same at 1024 (one wave of prep); 120 workers (d_k 64) 77 : 88 at
+    // 2048, 154 : 166; but 24 workers (32 heads) 309 : 76 at 1024.
+    // Otherwise the prep grid, then the scan.
     const int items = c->B * c->H * (c->dv / p.dv_slice);
     const int workers = c->num_sms - items;
-    const bool fuse = c->gdn_fuse && p.dv_slice <= 32 && 3 * workers >= 2 * c->num_sms && chunks * c->H > 2 * c->num_sms;
+    const bool fuse = c->gdn_fuse && p.dv_slice <= 32 && 2 * workers >= c->num_sms && chunks * c->H > 2 * c->num_sms;
     if (c->gdn_chain && c->gdn_snap && p.dv_slice == 32) {
         // state-chain form: the chain carries only S (one MMA batch a chunk),
         // the outputs follow in a parallel pass over per-chunk snapshots
