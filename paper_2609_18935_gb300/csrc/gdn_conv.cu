@@ -59,6 +59,9 @@ __device__ __forceinline__ void unpack8(const uint4& v, f2* x) {
     }
 }
 
+// ALIGNED: the inputs lie on the 16-byte grid; otherwise their channels are read
+// one by one.
+template <bool ALIGNED>
 __global__ void __launch_bounds__(kThreads, 4) gdn_conv_kernel(const __grid_constant__ ConvParams p) {
     const int g = blockIdx.x * kThreads + threadIdx.x;       // channels 8 g .. 8 g + 7
     const bool act = 8 * g < p.channels;
@@ -69,7 +72,15 @@ __global__ void __launch_bounds__(kThreads, 4) gdn_conv_kernel(const __grid_cons
     const int64_t stride = c < 2 * hk ? hk : p.H * p.dv;
     const __nv_bfloat16* in = (c < hk ? p.xq : c < 2 * hk ? p.xk : p.xv) + (c - first);
     __nv_bfloat16* out = (c < hk ? p.yq : c < 2 * hk ? p.yk : p.yv) + (c - first);
-    auto row = [&](int64_t tok) { return *reinterpret_cast<const uint4*>(in + tok * stride); };
+    auto row = [&](int64_t tok) {
+        const __nv_bfloat16* x = in + tok * stride;
+        if constexpr (ALIGNED) return *reinterpret_cast<const uint4*>(x);
+        uint4 v;
+        __nv_bfloat16* e = reinterpret_cast<__nv_bfloat16*>(&v);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e[i] = x[i];
+        return v;
+    };
     auto old_row = [&](int b, int r) {
         return *reinterpret_cast<const uint4*>(p.state_in + ((int64_t)b * 3 + r) * p.channels + c);
     };
@@ -170,8 +181,8 @@ __global__ void __launch_bounds__(kThreads, 4) gdn_conv_kernel(const __grid_cons
 
 void launch_gdn_conv(const ConvParams& p, cudaStream_t s) {
     if (p.total <= 0) return;
-    launch_pdl(gdn_conv_kernel, dim3((p.channels / 8 + kThreads - 1) / kThreads, p.n_strips + p.n_chars), dim3(kThreads),
-               0, s, p);
+    launch_pdl(p.aligned ? gdn_conv_kernel<true> : gdn_conv_kernel<false>,
+               dim3((p.channels / 8 + kThreads - 1) / kThreads, p.n_strips + p.n_chars), dim3(kThreads), 0, s, p);
 }
 
 }  // namespace kvm

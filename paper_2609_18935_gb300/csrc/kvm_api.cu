@@ -1181,7 +1181,7 @@ kvm_status do_attention(kvm_ctx* c, int layer, const int32_t* tail_cu, const voi
             st.slot0 = pl.cta_tile[c0] == t ? 2 * c0 : 2 * c0 + 1;
             st.token0 = tail_cu[b] + tok;
             st.rows = (int16_t)(std::min(p.tok_per_tile, Ms[b] - tok) * c->g);
-            st.head0 = (int16_t)(local / pl.n_qtiles[b] * c->g);
+            st.head0 = local / pl.n_qtiles[b] * c->g;
         }
         ps = prof_begin(c, KVM_K_ATTN_COMBINE, s);
         launch_attn_combine(cp, s);
@@ -1221,7 +1221,10 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     // its blocks each convolve their head's q and k themselves: cheaper than a
     // launch for a few tokens (one character's decode step 4.0 against 4.4 us,
     // 32 characters' 15.6 against 16.4; at 4 tokens 6.4 : 7.5 and 25 : 21)
-    const bool conv_inside = c->conv && recur && (longest <= 2 || (longest <= 4 && total <= 32));
+    // inputs of the convolution may lie off the 16-byte grid (its own launch reads
+    // them channel by channel then)
+    const bool aligned = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
+    const bool conv_inside = c->conv && recur && aligned && (longest <= 2 || (longest <= 4 && total <= 32));
     if (c->conv && !conv_inside) {
         // short convolution + SiLU (+ k normalisation) from the carried conv
         // state; the delta rule then reads the convolved q, k, v
@@ -1235,7 +1238,9 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         // and strip) fill the SMs, at least 4
         cp.strip = 32;
         while (cp.strip > 4 && (int64_t)total * (c->conv_ch / 8) / cp.strip < 1024 * (int64_t)c->num_sms) cp.strip /= 2;
+        cp.strip = std::max(cp.strip, (total + 32767) / 32768);         // the grid's y extent
         cp.n_strips = (total + cp.strip - 1) / cp.strip;
+        cp.aligned = aligned;
         for (int b = 0; b <= c->B; ++b) cp.tail_cu[b] = tail_cu[b];
         cp.xq = static_cast<const __nv_bfloat16*>(q);
         cp.xk = static_cast<const __nv_bfloat16*>(k);

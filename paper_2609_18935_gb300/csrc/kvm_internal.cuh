@@ -172,8 +172,8 @@ struct AttnParams {
 struct SplitTile {
     int32_t slot0;
     int32_t token0;
-    int16_t block0, n_parts;
-    int16_t rows, head0;
+    int32_t head0;
+    int16_t block0, n_parts, rows;
 };
 struct CombineParams {
     int32_t Hq, D, g;
@@ -285,6 +285,7 @@ struct ConvParams {
     int32_t n_chars, H, dk, dv, channels;     // channels = H (2 d_k + d_v)
     int32_t total;                            // sum M
     int32_t strip, n_strips;                  // packed tokens a thread walks; ceil(total / strip)
+    int32_t aligned;                          // xq, xk, xv on 16 bytes
     int32_t tail_cu[kMaxChars + 1];
     const __nv_bfloat16* xq;                  // caller's pre-conv inputs [sum M][H][d_k]
     const __nv_bfloat16* xk;

@@ -72,3 +72,34 @@ def test_fork_carries_the_conv_state():
     for p in (pair, task):
         span_cu, sb, se, tails = W.round_plan(w, 1, [p.ctx.get_live(0)[0]])
         _ok(p.run_round(span_cu, sb, se, tails, W.tail_inputs(w, 1, tails)), "after fork")
+
+
+@pytest.mark.parametrize("tails", [[3, 1], [70, 33]])
+def test_conv_inputs_off_the_vector_grid(tails):
+    """The same values from buffers on and off the 16-byte grid."""
+    import torch
+    from paper_2609_18935_gb300 import kvm
+    H, D, n = 3, 64, sum(tails)
+    g = torch.Generator("cuda").manual_seed(4)
+    x = [torch.randn((n, H, D), generator=g, device="cuda").bfloat16() for _ in range(3)]
+    al, be = (torch.sigmoid(torch.randn((n, H), generator=g, device="cuda")) for _ in range(2))
+    w = torch.randn((3 * H * D, 4), generator=g, device="cuda")
+    got = []
+    for off in (0, 1, 3):
+        ctx = kvm.Context([kvm.LAYER_GDN], 8, 2, 64, 64, 1e4, H, D, D, [64, 64], n, conv_kernel=4)
+        ctx.set_conv_weights(0, w)
+        y = [torch.cat([t.new_zeros(off), t.flatten()])[off:].view(n, H, D) for t in x]
+        assert off == 0 or any(t.data_ptr() % 16 for t in y)
+        out = torch.empty_like(x[2])
+        ctx.gdn_chunk_scan_from_state(0, np.concatenate([[0], np.cumsum(tails)]), *y, al, be, out)
+        ctx.check()
+        got.append((out.float(), ctx.get_state(0), ctx.get_conv_state(0).float()))
+    for other in got[1:]:
+        assert torch.equal(got[0][2], other[2])
+        for a, b in zip(got[0][:2], other[:2]):
+            if max(tails) > 4:
+                assert torch.equal(a, b)
+            else:
+                # in a step the aligned inputs are convolved by the step itself, which
+                # sums k's norm in another order: a key moves by a rounding of bf16, 2^-8
+                assert (a - b).norm() <= 2.0 ** -8 * a.norm()
