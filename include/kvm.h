@@ -256,7 +256,8 @@ kvm_status kvm_tail_attn_prefill(kvm_ctx* ctx, int32_t layer, const int32_t* tai
  *   S_t = alpha_t S_{t-1} (I - beta_t k_t k_t^T) + beta_t v_t k_t^T,
  *   o_t = S_t q_t,
  * computed in chunks of 64 tokens (WY/UT form) starting at the first tail
- * token.  S is updated in place in the context.
+ * token, or token by token when no character has more than 32 (d_k 64: 48).
+ * S is updated in place in the context.
  * q, k device [sum M][n_gdn_heads][d_k] bf16 (k expected unit-norm per head
  * but not required); v device [sum M][n_gdn_heads][d_v] bf16; alpha, beta
  * device [sum M][n_gdn_heads] fp32; out device [sum M][n_gdn_heads][d_v]
@@ -465,7 +466,7 @@ kvm_status kvm_check(kvm_ctx* ctx, void* stream);
  * within the library's accuracy).  Measured in a stack of delta-rule layers
  * (1024-token tail): the state chain takes 36 us against 52 for the full
  * chain, but its larger prep and the output pass make a layer 86 us against
- * 60, so it is off by default.
+ * 51, so it is off by default.  With it on, short tails take it too.
  * KVM_PLAN_GDN_FUSED: when a round has few characters and long tails, the
  * prep and the chain run in one launch, prep blocks publishing each chunk's
  * record through flags to the chain blocks; off: a prep launch, then the
