@@ -256,8 +256,10 @@ kvm_status kvm_tail_attn_prefill(kvm_ctx* ctx, int32_t layer, const int32_t* tai
  *   S_t = alpha_t S_{t-1} (I - beta_t k_t k_t^T) + beta_t v_t k_t^T,
  *   o_t = S_t q_t,
  * computed in chunks of 64 tokens (WY/UT form) starting at the first tail
- * token, or token by token when no character has more than 32 (d_k 64: 48).
- * S is updated in place in the context.
+ * token, or token by token when no character has more than 32 (d_k 64: 48)
+ * and out, unless it is v itself, does not overlie the inputs.
+ * S is updated in place in the context.  out may overlie any of the inputs:
+ * they are read before an output takes their place.
  * q, k device [sum M][n_gdn_heads][d_k] bf16 (k expected unit-norm per head
  * but not required); v device [sum M][n_gdn_heads][d_v] bf16; alpha, beta
  * device [sum M][n_gdn_heads] fp32; out device [sum M][n_gdn_heads][d_v]

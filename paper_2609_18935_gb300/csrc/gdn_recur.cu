@@ -6,6 +6,11 @@
 // (64 KB a head at d_k = d_v = 128); the chunked form spends a whole 64-token
 // chunk's products, a record in memory and two launches on them.
 //
+// out may be v itself: a block stores only the rows whose v it stages, after it
+// has staged them.  It may not otherwise overlie the inputs (all of a head's
+// blocks stage its q, k and gates, in no order): the caller takes the chunked
+// form for that.
+//
 // One block of four warps per (character, head, 16 NR rows of S).  Eight lanes
 // share a row: lane j holds the float4 groups j, j + 8, ... of NR rows in
 // registers from the first token to the last, so that S moves once, and a
@@ -132,7 +137,9 @@ __global__ void __launch_bounds__(kThreads) gdn_recur_kernel(const __grid_consta
     grid_dependents_launch();
 
     // the carried inputs after the tail, into the other state buffer (the
-    // blocks of slice 0 also carry the head's q and k channels)
+    // blocks of slice 0 also carry the head's q and k channels).  Called before
+    // the staging: out may be v itself, and no output is stored before the
+    // barriers behind the staging.
     auto carry = [&]() {
         __nv_bfloat16* nst = p.state_out + (int64_t)b * 3 * cs;
         const int per_row = ROWS / 8 + (blockIdx.x == 0 ? 2 * GK : 0);
@@ -164,6 +171,7 @@ __global__ void __launch_bounds__(kThreads) gdn_recur_kernel(const __grid_consta
             s[r][2 * i] = x.x;
             s[r][2 * i + 1] = x.y;
         }
+    if constexpr (CONV) carry();
 
     for (int t0 = 0; t0 < M; t0 += T) {
         const int nt = min(T, M - t0);
@@ -286,7 +294,6 @@ __global__ void __launch_bounds__(kThreads) gdn_recur_kernel(const __grid_consta
 #pragma unroll
         for (int i = 0; i < NP; ++i)
             *reinterpret_cast<ulonglong2*>(Sg + (int64_t)r * DK + 32 * i) = make_ulonglong2(s[r][2 * i], s[r][2 * i + 1]);
-    if constexpr (CONV) carry();
 }
 
 template <int DK, int NR, bool CONV>

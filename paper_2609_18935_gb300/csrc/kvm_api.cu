@@ -1217,14 +1217,32 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         active += m > 0;
         longest = std::max(longest, m);
     }
-    const bool recur = longest <= recur_tail(c->dk) && !c->gdn_chain;
+    // An out that overlies the inputs.  In separate launches every input is read
+    // before the first output is stored.  Otherwise blocks store outputs while
+    // others still read: the token-by-token form bears out == v, the one-launch
+    // form also out == q and out == k of rows as wide as v's (a chunk's outputs
+    // follow its own record), each only at the same address.  The separate
+    // convolution leaves the gates as the caller's only inputs of what follows it.
+    auto meets = [&](const void* x, size_t bytes) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(x), o = reinterpret_cast<uintptr_t>(out);
+        return a < o + (size_t)total * c->H * c->dv * 2 && o < a + bytes;
+    };
+    const size_t rows = (size_t)total * c->H;
+    const bool on_gates = meets(alpha, rows * 4) || meets(beta, rows * 4);
+    const bool on_q = meets(q, rows * c->dk * 2), on_k = meets(k, rows * c->dk * 2);
+    const bool on_v = out != v && meets(v, rows * c->dv * 2);
+    const bool same_width = c->dk == c->dv;
+    const bool askew = on_v || (on_q && !(out == q && same_width)) || (on_k && !(out == k && same_width));
+    const bool recur = longest <= recur_tail(c->dk) && !c->gdn_chain && !on_gates &&
+                       (c->conv || !(on_q || on_k || on_v));
     // its blocks each convolve their head's q and k themselves: cheaper than a
     // launch for a few tokens (one character's decode step 4.0 against 4.4 us,
     // 32 characters' 15.6 against 16.4; at 4 tokens 6.4 : 7.5 and 25 : 21)
     // inputs of the convolution may lie off the 16-byte grid (its own launch reads
     // them channel by channel then)
     const bool aligned = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
-    const bool conv_inside = c->conv && recur && aligned && (longest <= 2 || (longest <= 4 && total <= 32));
+    const bool conv_inside = c->conv && recur && aligned && !(on_q || on_k || on_v) &&
+                             (longest <= 2 || (longest <= 4 && total <= 32));
     if (c->conv && !conv_inside) {
         // short convolution + SiLU (+ k normalisation) from the carried conv
         // state; the delta rule then reads the convolved q, k, v
@@ -1338,7 +1356,8 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     // Otherwise the prep grid, then the scan.
     const int items = c->B * c->H * (c->dv / p.dv_slice);
     const int workers = c->num_sms - items;
-    const bool fuse = c->gdn_fuse && p.dv_slice <= 32 && 2 * workers >= c->num_sms && chunks * c->H > 2 * c->num_sms;
+    const bool fuse = c->gdn_fuse && p.dv_slice <= 32 && 2 * workers >= c->num_sms && chunks * c->H > 2 * c->num_sms &&
+                      !on_gates && (c->conv || !askew);
     if (c->gdn_chain && c->gdn_snap && p.dv_slice == 32) {
         // state-chain form: the chain carries only S (one MMA batch a chunk),
         // the outputs follow in a parallel pass over per-chunk snapshots

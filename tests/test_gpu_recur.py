@@ -96,3 +96,61 @@ def test_short_tails_after_the_convolution(heads, dk, dv):
                               W.tail_inputs(w, r, tails))
         bad = {k: v for k, v in errs.items() if not v <= 5e-3}       # the library's bar, bf16 inputs
         assert not bad, (r, bad)
+
+
+@pytest.mark.parametrize("conv", [False, True])
+@pytest.mark.parametrize("tails,over", [(t, o) for t in ([1, 0], [2, 1], [20, 1]) for o in ("v", "q", "k", "v_ahead", "gates")] +
+                         [([2048], "q"), ([2048], "q_ahead"), ([2048], "gates")])
+def test_outputs_over_the_inputs(tails, over, conv):
+    """An out that lies over an input, at its address or four rows before it:
+    outputs, state and carried convolution inputs as with an out of its own."""
+    import torch
+    from paper_2609_18935_gb300 import kvm
+    H, D, n, B = 16, 128, sum(tails), len(tails)
+    row = H * D
+    g = torch.Generator("cuda").manual_seed(8)
+    cu = np.concatenate([[0], np.cumsum(tails)])
+    x = [torch.randn((n, H, D), generator=g, device="cuda").bfloat16() for _ in range(3)]
+    x[1] = (x[1].float() / x[1].float().norm(dim=-1, keepdim=True)).bfloat16()
+    gates = torch.sigmoid(torch.randn((2, n, H), generator=g, device="cuda") + 1)
+    w = torch.randn((3 * row, 4), generator=g, device="cuda")
+    S = 0.2 * torch.randn((B, H, D, D), generator=g, device="cuda")
+    got = []
+    for shared in (False, True):
+        ctx = kvm.Context([kvm.LAYER_GDN], 8, 2, 64, 64, 1e4, H, D, D, [64] * B, n, conv_kernel=4 if conv else 0)
+        ctx.set_state(0, S)
+        if conv:
+            ctx.set_conv_weights(0, w)
+        # q, k, v, with room before each, and the gates inside out's bytes
+        y = []
+        for t in x:
+            room = torch.zeros(4 * row + t.numel(), dtype=torch.bfloat16, device="cuda")
+            room[4 * row:] = t.flatten()
+            y.append(room)
+        at = {"q": 0, "k": 1, "v": 2}.get(over[0])
+        al, be = gates.clone()
+        if over == "gates":
+            room = torch.zeros(n * row, dtype=torch.bfloat16, device="cuda")
+            al, be = (room[i * n * H * 2:(i + 1) * n * H * 2].view(torch.float32).view(n, H) for i in (0, 1))
+            al.copy_(gates[0])
+            be.copy_(gates[1])
+            out = room
+        else:
+            out = y[at][:n * row] if over.endswith("ahead") else y[at][4 * row:]
+        out = out.view(n, H, D) if shared else torch.empty((n, H, D), dtype=torch.bfloat16, device="cuda")
+        torch.cuda.synchronize()
+        q, k, v = (t[4 * row:].view(n, H, D) for t in y)
+        ctx.gdn_chunk_scan_from_state(0, cu, q, k, v, al, be, out)
+        ctx.check()
+        got.append((out.float(), ctx.get_state(0), ctx.get_conv_state(0).float() if conv else torch.zeros(1)))
+    (o, s, c), (o2, s2, c2) = got
+    assert torch.equal(c, c2)
+    if over == "v" or n > 2000:                    # the same kernels, or two forms that agree to the bit
+        assert torch.equal(o, o2) and torch.equal(s, s2)
+    else:
+        # the chunked form for the token-by-token one: an output rounds to bf16 once
+        # either way, states differ by the chunked form's 2e-5; a convolution in a
+        # launch of its own sums a key's norm in another order, which moves the key by a
+        # rounding of bf16, 2^-8
+        assert (o - o2).norm() <= 2.0 ** -7 * o.norm()
+        assert (s - s2).norm() <= (2.0 ** -8 if conv else 2e-5) * s.norm()
