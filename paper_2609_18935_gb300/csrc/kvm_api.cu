@@ -679,8 +679,19 @@ namespace {
 // Copies of the state accessors: `rows` pieces of `bytes` bytes each, a row
 // pitch on either side, of up to two arrays.  A kernel of the library follows
 // and precedes its neighbours with the overlapped launches of all the others
-// and costs the host a third of a memcpy call; memory of another device than
-// the current one, or off the 16-byte grid, goes through cudaMemcpy2DAsync.
+// and costs the host a third of a memcpy call.  Everything it cannot read or
+// write in place goes through cudaMemcpy2DAsync: memory that is not this
+// device's own (another GPU's, the host's, managed), buffers off the 16-byte
+// grid, calls made with another device current.
+bool own_memory(const kvm_ctx* c, const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == c->device;
+}
+
 kvm_status copy_state(kvm_ctx* c, void* const* dst, const void* const* src, int n, size_t dpitch, size_t spitch,
                       size_t bytes, int rows, cudaStream_t s) {
     if (!bytes || !rows) return KVM_OK;
@@ -688,7 +699,9 @@ kvm_status copy_state(kvm_ctx* c, void* const* dst, const void* const* src, int 
     CUDA_TRY(cudaGetDevice(&dev));
     uintptr_t bits = (uintptr_t)(rows > 1 ? dpitch | spitch : 0);
     for (int i = 0; i < n; ++i) bits |= reinterpret_cast<uintptr_t>(dst[i]) | reinterpret_cast<uintptr_t>(src[i]);
-    if (dev != c->device || (bits & 15)) {
+    bool own = dev == c->device && !(bits & 15);
+    for (int i = 0; i < n && own; ++i) own = own_memory(c, dst[i]) && own_memory(c, src[i]);
+    if (!own) {
         for (int i = 0; i < n; ++i)
             CUDA_TRY(rows > 1 ? cudaMemcpy2DAsync(dst[i], dpitch, src[i], spitch, bytes, rows, cudaMemcpyDeviceToDevice, s)
                               : cudaMemcpyAsync(dst[i], src[i], bytes, cudaMemcpyDeviceToDevice, s));

@@ -65,3 +65,47 @@ def test_reads_follow_the_writes_queued_before_them():
             sync()
         runs.append(got)
     assert all(torch.equal(a, b) for a, b in zip(*runs))
+
+
+def test_buffers_outside_the_device_are_copied_by_memcpy():
+    """Pinned host memory: no kernel of the library reads or writes it
+    (the launch count stays), the values arrive all the same."""
+    import torch
+    from paper_2609_18935_gb300 import kvm
+    H, D = 4, 64
+    ctx = kvm.Context([kvm.LAYER_GDN, kvm.LAYER_ATTN], 8, 2, 64, 64, 1e4, H, D, D, [128], 8)
+    ctx.load_prefix(0, 100, 100, np.arange(100, dtype=np.int32))
+    S = torch.randn((1, H, D, D)).pin_memory()
+    K, V = (torch.randn((2, 100, 64)).bfloat16().pin_memory() for _ in range(2))
+    back = [torch.zeros_like(t).pin_memory() for t in (S, K, V)]
+    lib, s = kvm._lib, torch.cuda.current_stream().cuda_stream
+    before = lib.kvm_launch_count(ctx._h)
+    for call in (lambda: lib.kvm_set_state(ctx._h, 0, S.data_ptr(), s),
+                 lambda: lib.kvm_set_kv(ctx._h, 1, 0, K.data_ptr(), V.data_ptr(), s),
+                 lambda: lib.kvm_get_state(ctx._h, 0, back[0].data_ptr(), s),
+                 lambda: lib.kvm_get_kv(ctx._h, 1, 0, back[1].data_ptr(), back[2].data_ptr(), s)):
+        assert call() == 0, lib.kvm_last_error().decode()
+    torch.cuda.synchronize()
+    assert lib.kvm_launch_count(ctx._h) == before
+    for a, b in zip((S, K, V), back):
+        assert torch.equal(a, b)
+    got = ctx.get_state(0)
+    assert lib.kvm_launch_count(ctx._h) == before + 1 and torch.equal(got.cpu(), S)
+
+
+def test_accessors_under_capture():
+    """A captured read replays with the state of the moment."""
+    import torch
+    from paper_2609_18935_gb300 import kvm
+    H, D = 4, 64
+    ctx = kvm.Context([kvm.LAYER_GDN], 8, 2, 64, 64, 1e4, H, D, D, [64], 8)
+    S = [torch.randn((1, H, D, D), device="cuda") for _ in range(2)]
+    ctx.set_state(0, S[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = ctx.get_state(0)
+    for x in S:
+        ctx.set_state(0, x)
+        graph.replay()
+        assert torch.equal(out, x)
