@@ -21,33 +21,13 @@
 // [state; tail]) into the other of two state buffers, so that no block reads
 // a state row that another block of the same launch writes.
 #include "kvm_internal.cuh"
+#include "packed_f32.cuh"
 
 namespace kvm {
 namespace {
 
 constexpr int kThreads = 128;
 constexpr int kAhead = 4;                    // rows loaded ahead of their use
-
-// the quotient to 2 ulp (the result is rounded to bf16)
-__device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.f + __expf(-x)); }
-
-using f2 = unsigned long long;               // two packed floats
-
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
 
 // Eight bf16 channels as four pairs of floats.
 __device__ __forceinline__ void unpack8(const uint4& v, f2* x) {
@@ -149,9 +129,9 @@ __global__ void __launch_bounds__(kThreads, 4) gdn_conv_kernel(const __grid_cons
                 f2 acc = 0;                                  // two zeros
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc = fma2(w[i][e], x[i][e], acc);
-                const float2 a = unpack2(acc);
-                y[2 * e] = silu(a.x);
-                y[2 * e + 1] = silu(a.y);
+                const float2 a = silu2(acc);
+                y[2 * e] = a.x;
+                y[2 * e + 1] = a.y;
             }
             if (any_k) {                                     // uniform per warp
                 float tot = 0.f;

@@ -28,35 +28,17 @@
 // token's k and q ahead, two accumulators per dot product, and carrying S / prod
 // alpha instead of decaying S were each slower (more registers, fewer blocks).
 #include "kvm_internal.cuh"
+#include "packed_f32.cuh"
 
 namespace kvm {
 namespace {
 
 constexpr int kThreads = 128;
 
-using f2 = unsigned long long;        // two packed floats
-
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
 __device__ __forceinline__ float sum2(f2 v) {
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-    return lo + hi;
+    const float2 x = unpack2(v);
+    return x.x + x.y;
 }
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 __device__ __forceinline__ void unpack8(const uint4& v, float* x) {
     const uint32_t* w = reinterpret_cast<const uint32_t*>(&v);
 #pragma unroll
@@ -84,7 +66,8 @@ struct Part {
         return *reinterpret_cast<const uint4*>(t >= 0 ? in + (int64_t)t * stride + c
                                                       : state + (int64_t)(t + 3) * state_stride + c);
     }
-    // convolution and SiLU of channels c .. c + 7 at token t, in gdn_conv_kernel's order
+    // convolution and SiLU of channels c .. c + 7 at token t, the taps in gdn_conv_kernel's order
+    // (a key's norm is summed in another)
     __device__ __forceinline__ void conv8(int t, int c, float* y) const {
         uint4 r[4];
 #pragma unroll
@@ -93,13 +76,17 @@ struct Part {
 #pragma unroll
         for (int i = 0; i < 4; ++i) unpack8(r[i], x[i]);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const float4 tap = *(reinterpret_cast<const float4*>(w) + c + e);
-            float acc = fmaf(tap.x, x[0][e], 0.f);
-            acc = fmaf(tap.y, x[1][e], acc);
-            acc = fmaf(tap.z, x[2][e], acc);
-            acc = fmaf(tap.w, x[3][e], acc);
-            y[e] = __fdividef(acc, 1.f + __expf(-acc));
+        for (int e = 0; e < 8; e += 2) {
+            f2 acc = 0;                              // two zeros
+            const float4 a = *(reinterpret_cast<const float4*>(w) + c + e);
+            const float4 b = *(reinterpret_cast<const float4*>(w) + c + e + 1);
+            acc = fma2(pack2(a.x, b.x), pack2(x[0][e], x[0][e + 1]), acc);
+            acc = fma2(pack2(a.y, b.y), pack2(x[1][e], x[1][e + 1]), acc);
+            acc = fma2(pack2(a.z, b.z), pack2(x[2][e], x[2][e + 1]), acc);
+            acc = fma2(pack2(a.w, b.w), pack2(x[3][e], x[3][e + 1]), acc);
+            const float2 v = silu2(acc);
+            y[e] = v.x;
+            y[e + 1] = v.y;
         }
     }
 };

@@ -103,3 +103,24 @@ def test_conv_inputs_off_the_vector_grid(tails):
                 # in a step the aligned inputs are convolved by the step itself, which
                 # sums k's norm in another order: a key moves by a rounding of bf16, 2^-8
                 assert (a - b).norm() <= 2.0 ** -8 * a.norm()
+
+
+@pytest.mark.parametrize("n,pre", [(n, x) for n in (1, 9, 70) for x in (-88.0, -87.5, -60.0, -0.75, 3.0, 300.0, -89.0)] +
+                         [(1, float("inf"))])
+def test_silu_over_its_range(n, pre):
+    """silu(x) = x / (1 + e^-x), which keeps its small values until e^-x passes the
+    largest float and is 0 from there (v of every token; keys of 1 / 8 in each of 64
+    dims): in the step, in a launch before the recurrence, and before the chunked form."""
+    import math
+    import torch
+    from paper_2609_18935_gb300 import kvm
+    H, D = 2, 64
+    ctx = kvm.Context([kvm.LAYER_GDN], 8, 2, 64, 64, 1e4, H, D, D, [64], n, conv_kernel=4)
+    w = torch.zeros((3 * H * D, 4), device="cuda")
+    w[:, 3] = 1
+    ctx.set_conv_weights(0, w)
+    one, gate = torch.ones((n, H, D), device="cuda").bfloat16(), torch.ones((n, H), device="cuda")
+    ctx.gdn_chunk_scan_from_state(0, [0, n], one, one, pre * one, gate, gate, torch.empty_like(one))
+    # v and the key round to bf16: 2^-9 each; __expf(88) is good to ~2^-16
+    want = np.full((1, H, D, D), pre / (1 + math.exp(-pre)) / 8 if pre > -88.7 else 0.0)
+    np.testing.assert_allclose(ctx.get_state(0).cpu().numpy(), want, rtol=2.0 ** -7, atol=0)
