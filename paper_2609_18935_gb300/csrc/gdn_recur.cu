@@ -6,10 +6,13 @@
 // (64 KB a head at d_k = d_v = 128); the chunked form spends a whole 64-token
 // chunk's products, a record in memory and two launches on them.
 //
-// out may be v itself: a block stores only the rows whose v it stages, after it
-// has staged them.  It may not otherwise overlie the inputs (all of a head's
-// blocks stage its q, k and gates, in no order): the caller takes the chunked
-// form for that.
+// Without the convolution out may be v itself: a block stores only rows whose v
+// it has staged, and no other block reads those.  It may not otherwise overlie the
+// inputs (all blocks of a head stage its q, k and gates, in no order; a convolved
+// step reads inputs once more after its outputs, to carry them): the caller
+// convolves in a launch of its own or takes the chunked form for that.  Carrying v
+// ahead of the outputs instead, in registers or stored at once, made a convolved
+// step of 8 characters slower (2 tokens 4.8 -> 5.9, 4 tokens 6.7 -> 8.5 us).
 //
 // One block of four warps per (character, head, 16 NR rows of S).  Eight lanes
 // share a row: lane j holds the float4 groups j, j + 8, ... of NR rows in
@@ -36,8 +39,9 @@ namespace {
 constexpr int kThreads = 128;
 
 __device__ __forceinline__ float sum2(f2 v) {
-    const float2 x = unpack2(v);
-    return x.x + x.y;
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    return lo + hi;
 }
 __device__ __forceinline__ void unpack8(const uint4& v, float* x) {
     const uint32_t* w = reinterpret_cast<const uint32_t*>(&v);
@@ -66,8 +70,8 @@ struct Part {
         return *reinterpret_cast<const uint4*>(t >= 0 ? in + (int64_t)t * stride + c
                                                       : state + (int64_t)(t + 3) * state_stride + c);
     }
-    // convolution and SiLU of channels c .. c + 7 at token t, the taps in gdn_conv_kernel's order
-    // (a key's norm is summed in another)
+    // convolution and SiLU of channels c .. c + 7 at token t, the taps in gdn_conv_kernel's
+    // order (a key's norm is summed in another)
     __device__ __forceinline__ void conv8(int t, int c, float* y) const {
         uint4 r[4];
 #pragma unroll
@@ -76,15 +80,17 @@ struct Part {
 #pragma unroll
         for (int i = 0; i < 4; ++i) unpack8(r[i], x[i]);
 #pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float4 tap = *(reinterpret_cast<const float4*>(w) + c + e);
+            float acc = fmaf(tap.x, x[0][e], 0.f);
+            acc = fmaf(tap.y, x[1][e], acc);
+            acc = fmaf(tap.z, x[2][e], acc);
+            acc = fmaf(tap.w, x[3][e], acc);
+            y[e] = acc;
+        }
+#pragma unroll
         for (int e = 0; e < 8; e += 2) {
-            f2 acc = 0;                              // two zeros
-            const float4 a = *(reinterpret_cast<const float4*>(w) + c + e);
-            const float4 b = *(reinterpret_cast<const float4*>(w) + c + e + 1);
-            acc = fma2(pack2(a.x, b.x), pack2(x[0][e], x[0][e + 1]), acc);
-            acc = fma2(pack2(a.y, b.y), pack2(x[1][e], x[1][e + 1]), acc);
-            acc = fma2(pack2(a.z, b.z), pack2(x[2][e], x[2][e + 1]), acc);
-            acc = fma2(pack2(a.w, b.w), pack2(x[3][e], x[3][e + 1]), acc);
-            const float2 v = silu2(acc);
+            const float2 v = silu2(pack2(y[e], y[e + 1]));
             y[e] = v.x;
             y[e + 1] = v.y;
         }
@@ -124,9 +130,7 @@ __global__ void __launch_bounds__(kThreads) gdn_recur_kernel(const __grid_consta
     grid_dependents_launch();
 
     // the carried inputs after the tail, into the other state buffer (the
-    // blocks of slice 0 also carry the head's q and k channels).  Called before
-    // the staging: out may be v itself, and no output is stored before the
-    // barriers behind the staging.
+    // blocks of slice 0 also carry the head's q and k channels)
     auto carry = [&]() {
         __nv_bfloat16* nst = p.state_out + (int64_t)b * 3 * cs;
         const int per_row = ROWS / 8 + (blockIdx.x == 0 ? 2 * GK : 0);
@@ -158,7 +162,6 @@ __global__ void __launch_bounds__(kThreads) gdn_recur_kernel(const __grid_consta
             s[r][2 * i] = x.x;
             s[r][2 * i + 1] = x.y;
         }
-    if constexpr (CONV) carry();
 
     for (int t0 = 0; t0 < M; t0 += T) {
         const int nt = min(T, M - t0);
@@ -281,6 +284,7 @@ __global__ void __launch_bounds__(kThreads) gdn_recur_kernel(const __grid_consta
 #pragma unroll
         for (int i = 0; i < NP; ++i)
             *reinterpret_cast<ulonglong2*>(Sg + (int64_t)r * DK + 32 * i) = make_ulonglong2(s[r][2 * i], s[r][2 * i + 1]);
+    if constexpr (CONV) carry();
 }
 
 template <int DK, int NR, bool CONV>

@@ -1232,10 +1232,11 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     }
     // An out that overlies the inputs.  In separate launches every input is read
     // before the first output is stored.  Otherwise blocks store outputs while
-    // others still read: the token-by-token form bears out == v, the one-launch
-    // form also out == q and out == k of rows as wide as v's (a chunk's outputs
-    // follow its own record), each only at the same address.  The separate
-    // convolution leaves the gates as the caller's only inputs of what follows it.
+    // others still read: the token-by-token form without the convolution bears
+    // out == v, the one-launch form also out == q and out == k of rows as wide as
+    // v's (a chunk's outputs follow its own record), each only at the same address.
+    // The separate convolution leaves the gates as the caller's only inputs of what
+    // follows it.
     auto meets = [&](const void* x, size_t bytes) {
         const uintptr_t a = reinterpret_cast<uintptr_t>(x), o = reinterpret_cast<uintptr_t>(out);
         return a < o + (size_t)total * c->H * c->dv * 2 && o < a + bytes;
@@ -1254,7 +1255,7 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     // inputs of the convolution may lie off the 16-byte grid (its own launch reads
     // them channel by channel then)
     const bool aligned = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
-    const bool conv_inside = c->conv && recur && aligned && !(on_q || on_k || on_v) &&
+    const bool conv_inside = c->conv && recur && aligned && !(on_q || on_k || on_v || out == v) &&
                              (longest <= 2 || (longest <= 4 && total <= 32));
     if (c->conv && !conv_inside) {
         // short convolution + SiLU (+ k normalisation) from the carried conv

@@ -145,7 +145,7 @@ def test_outputs_over_the_inputs(tails, over, conv):
         got.append((out.float(), ctx.get_state(0), ctx.get_conv_state(0).float() if conv else torch.zeros(1)))
     (o, s, c), (o2, s2, c2) = got
     assert torch.equal(c, c2)
-    if over == "v" or n > 2000:                    # the same kernels, or two forms that agree to the bit
+    if (over == "v" and (not conv or max(tails) > 4)) or n > 2000:      # the same kernels, or two forms that agree to the bit
         assert torch.equal(o, o2) and torch.equal(s, s2)
     else:
         # the chunked form for the token-by-token one: an output rounds to bf16 once
