@@ -459,7 +459,8 @@ kvm_status kvm_check(kvm_ctx* ctx, void* stream);
 
 /* Launch plans of the delta-rule layers (no paper counterpart; fused
  * defaults to on, state chain to off).
- * KVM_PLAN_GDN_STATE_CHAIN (d_k = d_v = 128, one or few characters): the
+ * KVM_PLAN_GDN_STATE_CHAIN (d_k = d_v = 128, few enough characters that a
+ * block holds 32 rows of a head's state; nothing changes elsewhere): the
  * serial chunk chain carries only the state, S^T <- P_c S^T + B_c with
  * P_c = G_C I - K^T diag(w) W and B_c = K^T diag(w) U formed in the
  * parallel prep, and the chunks' outputs O = A U + Q' S0^T follow in one

@@ -1247,7 +1247,15 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     const bool on_v = out != v && meets(v, rows * c->dv * 2);
     const bool same_width = c->dk == c->dv;
     const bool askew = on_v || (on_q && !(out == q && same_width)) || (on_k && !(out == k && same_width));
-    const bool recur = longest <= recur_tail(c->dk) && !c->gdn_chain && !on_gates &&
+    // d_v rows of a head's state per scan block: split the rows (down to 32)
+    // until the (character, head, slice) blocks cover the SMs
+    int slices = 1;
+    while (c->dv / (2 * slices) >= 32 && c->dv % (2 * slices * 32) == 0 &&
+           (int64_t)active * c->H * slices < c->num_sms)
+        slices *= 2;
+    const int dv_slice = c->dv / slices;
+    const bool chain = c->gdn_chain && c->gdn_snap && dv_slice == 32;   // the state-chain form, where it is switched on
+    const bool recur = longest <= recur_tail(c->dk) && !chain && !on_gates &&
                        (c->conv || !(on_q || on_k || on_v));
     // its blocks each convolve their head's q and k themselves: cheaper than a
     // launch for a few tokens (one character's decode step 4.0 against 4.4 us,
@@ -1325,15 +1333,7 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     std::memset(&p, 0, sizeof p);
     p.n_chars = c->B;
     p.H = c->H; p.dk = c->dk; p.dv = c->dv;
-    // d_v rows of a head's state per scan block: split the rows (down to 32)
-    // until the (character, head, slice) blocks cover the SMs
-    {
-        int slices = 1;
-        while (c->dv / (2 * slices) >= 32 && c->dv % (2 * slices * 32) == 0 &&
-               (int64_t)active * c->H * slices < c->num_sms)
-            slices *= 2;
-        p.dv_slice = c->dv / slices;
-    }
+    p.dv_slice = dv_slice;
     p.q = static_cast<const __nv_bfloat16*>(q);
     p.k = static_cast<const __nv_bfloat16*>(k);
     p.v = static_cast<const __nv_bfloat16*>(v);
@@ -1372,7 +1372,7 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     const int workers = c->num_sms - items;
     const bool fuse = c->gdn_fuse && p.dv_slice <= 32 && 2 * workers >= c->num_sms && chunks * c->H > 2 * c->num_sms &&
                       !on_gates && (c->conv || !askew);
-    if (c->gdn_chain && c->gdn_snap && p.dv_slice == 32) {
+    if (chain) {
         // state-chain form: the chain carries only S (one MMA batch a chunk),
         // the outputs follow in a parallel pass over per-chunk snapshots
         p.snap = c->gdn_snap;
@@ -1384,6 +1384,7 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         const cudaError_t e = launch_gdn_v2(p, fuse ? std::min(c->num_sms, items + chunks * c->H) : 0, s);
         prof_end(c, ps, s);
         if (e == cudaSuccess) {
+            c->launches += fuse ? 1 : 2;              // prof_begin counted one of them
             LAUNCH_CHECK(c);
             return KVM_OK;
         }
@@ -1393,6 +1394,7 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
         const cudaError_t e2 = launch_gdn_v2(p, 0, s);
         prof_end(c, ps2, s);
         if (e2 != cudaSuccess) return fail(KVM_E_CUDA, "delta-rule launch failed: %s", cudaGetErrorString(e2));
+        c->launches += 2;
         LAUNCH_CHECK(c);
         return KVM_OK;
     }

@@ -154,3 +154,31 @@ def test_outputs_over_the_inputs(tails, over, conv):
         # rounding of bf16, 2^-8
         assert (o - o2).norm() <= 2.0 ** -7 * o.norm()
         assert (s - s2).norm() <= (2.0 ** -8 if conv else 2e-5) * s.norm()
+
+
+@pytest.mark.parametrize("heads,dk,B,launches", [(16, 128, 1, 3), (16, 128, 16, 1), (16, 64, 1, 1)])
+def test_a_decode_step_with_the_state_chain_on(heads, dk, B, launches):
+    """The state chain takes a short tail where it can be served (prep, chain and
+    outputs); elsewhere the switch changes nothing (one launch, the same bits)."""
+    import torch
+    from paper_2609_18935_gb300 import kvm
+    g = torch.Generator("cuda").manual_seed(9)
+    r = lambda *s: torch.randn(s, generator=g, device="cuda")
+    q, k, v = r(B, heads, dk).bfloat16(), (r(B, heads, dk) / dk ** 0.5).bfloat16(), r(B, heads, dk).bfloat16()
+    al, be, S = torch.sigmoid(r(B, heads)), torch.sigmoid(r(B, heads)), r(B, heads, dk, dk)
+    got = []
+    for on in (False, True):
+        ctx = kvm.Context([kvm.LAYER_GDN], 8, 2, 64, 64, 1e4, heads, dk, dk, [64] * B, B)
+        ctx.set_gdn_state_chain(on)
+        ctx.set_state(0, S)
+        out = torch.empty_like(v)
+        before = kvm._lib.kvm_launch_count(ctx._h)
+        ctx.gdn_chunk_scan_from_state(0, np.arange(B + 1), q, k, v, al, be, out)
+        n = kvm._lib.kvm_launch_count(ctx._h) - before
+        ctx.check()
+        got.append((out.float(), ctx.get_state(0)))
+    assert n == launches
+    if n == 1:
+        assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    else:
+        assert (got[0][1] - got[1][1]).norm() <= 2e-5 * got[0][1].norm()
