@@ -1,6 +1,7 @@
 """Two rounds of a stack of one delta-rule layer with nothing between them: the
 second round's launch may start before the first has finished, and must still
-read the state the first one wrote."""
+read the state the first one wrote: as one launch for prep and scan (long tails),
+as two, and token by token."""
 import numpy as np
 import pytest
 
@@ -9,8 +10,9 @@ from workload import synth as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("heads,dk,tail", [(16, 128, 1024), (4, 64, 4096), (16, 128, 256), (16, 128, 1)])
-def test_rounds_in_a_row_carry_the_state(heads, dk, tail):
+@pytest.mark.parametrize("heads,dk,tail,launches", [(16, 128, 2048, 1), (4, 64, 8192, 1), (16, 128, 1024, 2),
+                                                    (4, 64, 4096, 2), (16, 128, 256, 2), (16, 128, 1, 1)])
+def test_rounds_in_a_row_carry_the_state(heads, dk, tail, launches):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -25,10 +27,12 @@ def test_rounds_in_a_row_carry_the_state(heads, dk, tail):
         ctx.set_state(0, S)
         outs = [torch.empty((tail, heads, dk), dtype=torch.bfloat16, device="cuda") for _ in range(4)]
         torch.cuda.synchronize()
+        before = kvm._lib.kvm_launch_count(ctx._h)
         for out in outs:
             ctx.gdn_chunk_scan_from_state(0, [0, tail], x["q"], x["k"], x["v"], x["alpha"], x["beta"], out)
             if wait:
                 torch.cuda.synchronize()
+        assert kvm._lib.kvm_launch_count(ctx._h) - before == launches * len(outs)    # the form this size is here for
         got.append([o.view(torch.int16) for o in outs] + [ctx.get_state(0)])
         ctx.check()
     for a, b in zip(*got):

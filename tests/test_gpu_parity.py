@@ -266,12 +266,13 @@ def test_host_resident_round_equals_device_round(arena):
 
 
 @pytest.mark.parametrize("state_chain", [True, False])
-@pytest.mark.parametrize("n_chars,tails", [(1, [256]), (1, [1024]), (2, [130, 64]), (1, [1])])
-def test_delta_rule_launch_plans_agree(n_chars, tails, state_chain):
+@pytest.mark.parametrize("n_chars,tails,fuses", [(1, [256], False), (1, [1024], False), (1, [1281], True), (1, [2048], True),
+                                                 (2, [130, 64], False), (1, [1], False)])
+def test_delta_rule_launch_plans_agree(n_chars, tails, fuses, state_chain):
     """The delta-rule layer as one launch (prep workers publishing records
     to chain blocks in the same grid) and as separate launches run the same
     arithmetic: outputs and states bit-identical, over two rounds, in both
-    forms of the chain."""
+    forms of the chain.  `fuses`: whether this size takes the one launch."""
     import torch
     from paper_2609_18935_gb300 import kvm
     shape = W.ModelShape([W.GDN, W.GDN], 16, 2, 256, 64, 1e4, 16, 128, 128)
@@ -291,8 +292,11 @@ def test_delta_rule_launch_plans_agree(n_chars, tails, state_chain):
         ins = W.device_round_inputs(w, 900 + r, tails)
         outs = [{l: torch.empty((sum(tails), 16, 128), dtype=torch.bfloat16, device="cuda") for l in (0, 1)}
                 for _ in range(2)]
+        n = [kvm._lib.kvm_launch_count(ctx._h) for ctx in (a, b)]
         a.update_round(z, [], [], tail_cu, ins, outs[0])
         b.update_round(z, [], [], tail_cu, ins, outs[1])
+        na, nb = (kvm._lib.kvm_launch_count(ctx._h) - x for ctx, x in zip((a, b), n))
+        assert nb - na == (2 if fuses else 0)       # one launch fewer in each of two layers
         a.check()
         b.check()
         for l in (0, 1):
