@@ -185,7 +185,7 @@ kvm_status kvm_plan_spans_from_positions(int32_t live, const int32_t* positions,
                                          const int64_t* pos_begin, const int64_t* pos_end,
                                          int32_t* span_begin, int32_t* span_end);
 
-/* The work partition kvm_tail_attn_prefill uses for one attention layer
+/* The attention's work, cut evenly, for one attention layer
  * (Eq. 3), for live lengths L'_b live host [n_chars] (after removal) and
  * tails tail_cu host [n_chars+1].  Query tiles hold 128 / g tail tokens of
  * one KV head (g = n_q_heads / n_kv_heads) and are numbered (character, KV
@@ -197,14 +197,26 @@ kvm_status kvm_plan_spans_from_positions(int32_t live, const int32_t* positions,
  * [max_blocks + 1].  *n_tiles = number of query tiles.  split_first_block
  * host [max_blocks]: for each of the *n_split query tiles that several
  * blocks share, the first block that starts inside it (its partials are
- * merged by the combine kernel).  kvm_tail_attn_prefill uses max_blocks =
- * min(320, the device's SM count); with more than a wave and a half of query
- * tiles it first deals whole tiles to the blocks in waves and cuts only the
- * rest in this way, and tiles of at most 5 key tiles get a block each.  Errors: KVM_E_INVAL, KVM_E_UNSUPPORTED. */
+ * merged by the combine kernel).  Errors: KVM_E_INVAL, KVM_E_UNSUPPORTED. */
 kvm_status kvm_plan_attention(int32_t n_chars, const int32_t* live, const int32_t* tail_cu,
                               int32_t n_q_heads, int32_t n_kv_heads, int32_t max_blocks,
                               int32_t* n_blocks, int32_t* n_tiles, int32_t* block_tile,
                               int32_t* block_key, int32_t* n_split, int32_t* split_first_block);
+
+/* The partition kvm_tail_attn_prefill launches, with max_blocks = min(320,
+ * the device's SM count): as kvm_plan_attention, but
+ *  - query tiles 0 .. *n_waves * *n_blocks - 1 are dealt whole, tile
+ *    w * *n_blocks + i to block i in an even wave w, to block
+ *    *n_blocks - 1 - i in an odd one, and only the tiles after them are cut.
+ *    There are waves while more than a wave and a half of tiles is left and no
+ *    block's dealt work passes its even share of all of it;
+ *  - when every query tile has at most 5 key tiles, and there are no more query
+ *    tiles than max_blocks, each gets a block (no waves, nothing shared). */
+kvm_status kvm_plan_attention_launch(int32_t n_chars, const int32_t* live, const int32_t* tail_cu,
+                                     int32_t n_q_heads, int32_t n_kv_heads, int32_t max_blocks,
+                                     int32_t* n_waves, int32_t* n_blocks, int32_t* n_tiles,
+                                     int32_t* block_tile, int32_t* block_key, int32_t* n_split,
+                                     int32_t* split_first_block);
 
 /* Partition of a character population over ranks (one GPU per rank):
  * characters are independent, so each rank maintains its own share with no

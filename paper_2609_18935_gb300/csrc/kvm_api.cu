@@ -866,10 +866,12 @@ extern "C" kvm_status kvm_plan_removal(int32_t n_chars, const int32_t* live, con
     return KVM_OK;
 }
 
-extern "C" kvm_status kvm_plan_attention(int32_t n_chars, const int32_t* live, const int32_t* tail_cu,
-                                         int32_t n_q_heads, int32_t n_kv_heads, int32_t max_blocks,
-                                         int32_t* n_blocks, int32_t* n_tiles, int32_t* block_tile,
-                                         int32_t* block_key, int32_t* n_split, int32_t* split_first_block) {
+namespace {
+// Both exported planners: the cut of all units (n_waves NULL), or the layer's own plan.
+kvm_status plan_attention_out(int32_t n_chars, const int32_t* live, const int32_t* tail_cu, int32_t n_q_heads,
+                              int32_t n_kv_heads, int32_t max_blocks, int32_t* n_waves, int32_t* n_blocks,
+                              int32_t* n_tiles, int32_t* block_tile, int32_t* block_key, int32_t* n_split,
+                              int32_t* split_first_block) {
     if (n_chars <= 0 || n_chars > kMaxChars) return fail(KVM_E_INVAL, "n_chars must be in [1,%d]", kMaxChars);
     if (!live || !tail_cu || !n_blocks || !n_tiles || !block_tile || !block_key || !n_split || !split_first_block)
         return fail(KVM_E_INVAL, "NULL argument");
@@ -887,7 +889,8 @@ extern "C" kvm_status kvm_plan_attention(int32_t n_chars, const int32_t* live, c
         if (L[b] < 0) return fail(KVM_E_INVAL, "negative live length at character %d", b);
     }
     AttnPlan pl;
-    plan_attention(n_chars, L.data(), M.data(), n_kv_heads, kAttnRows / g, max_blocks, false, pl);
+    plan_attention(n_chars, L.data(), M.data(), n_kv_heads, kAttnRows / g, max_blocks, n_waves != nullptr, pl);
+    if (n_waves) *n_waves = pl.waves;
     *n_blocks = pl.n_ctas;
     *n_tiles = pl.n_tiles;
     std::copy(pl.cta_tile.begin(), pl.cta_tile.end(), block_tile);
@@ -895,6 +898,25 @@ extern "C" kvm_status kvm_plan_attention(int32_t n_chars, const int32_t* live, c
     *n_split = (int32_t)pl.split_cb.size();
     std::copy(pl.split_cb.begin(), pl.split_cb.end(), split_first_block);
     return KVM_OK;
+}
+}  // namespace
+
+extern "C" kvm_status kvm_plan_attention(int32_t n_chars, const int32_t* live, const int32_t* tail_cu,
+                                         int32_t n_q_heads, int32_t n_kv_heads, int32_t max_blocks,
+                                         int32_t* n_blocks, int32_t* n_tiles, int32_t* block_tile,
+                                         int32_t* block_key, int32_t* n_split, int32_t* split_first_block) {
+    return plan_attention_out(n_chars, live, tail_cu, n_q_heads, n_kv_heads, max_blocks, nullptr, n_blocks, n_tiles,
+                              block_tile, block_key, n_split, split_first_block);
+}
+
+extern "C" kvm_status kvm_plan_attention_launch(int32_t n_chars, const int32_t* live, const int32_t* tail_cu,
+                                                int32_t n_q_heads, int32_t n_kv_heads, int32_t max_blocks,
+                                                int32_t* n_waves, int32_t* n_blocks, int32_t* n_tiles,
+                                                int32_t* block_tile, int32_t* block_key, int32_t* n_split,
+                                                int32_t* split_first_block) {
+    if (!n_waves) return fail(KVM_E_INVAL, "NULL argument");
+    return plan_attention_out(n_chars, live, tail_cu, n_q_heads, n_kv_heads, max_blocks, n_waves, n_blocks, n_tiles,
+                              block_tile, block_key, n_split, split_first_block);
 }
 
 extern "C" kvm_status kvm_plan_partition(int32_t n_chars, const int64_t* cost, int32_t n_ranks, int32_t* rank_of,

@@ -102,6 +102,10 @@ _SIGS = {
     "kvm_plan_attention": (C.c_int, [C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.c_int32, C.c_int32,
                                      C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                      C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
+    "kvm_plan_attention_launch": (C.c_int, [C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.c_int32, C.c_int32,
+                                            C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
+                                            C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32),
+                                            C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "kvm_plan_partition": (C.c_int, [C.c_int32, C.POINTER(C.c_int64), C.c_int32, C.POINTER(C.c_int32),
                                      C.POINTER(C.c_int64)]),
     "kvm_kv_compact_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_int64, C.c_int32,
@@ -288,17 +292,29 @@ def plan_spans_from_positions(positions, pos_begin, pos_end):
 
 
 def plan_attention(live, tail_cu, n_q_heads, n_kv_heads, max_blocks):
-    """kvm_plan_attention: the attention's work partition for one layer."""
+    """kvm_plan_attention: the attention's work for one layer, cut evenly."""
+    return _plan_attention(live, tail_cu, n_q_heads, n_kv_heads, max_blocks, False)
+
+
+def plan_attention_launch(live, tail_cu, n_q_heads, n_kv_heads, max_blocks):
+    """kvm_plan_attention_launch: the partition the layer runs, with "n_waves" of
+    whole query tiles dealt before the cut."""
+    return _plan_attention(live, tail_cu, n_q_heads, n_kv_heads, max_blocks, True)
+
+
+def _plan_attention(live, tail_cu, n_q_heads, n_kv_heads, max_blocks, launch):
     load_library()
     L, cu = _i32(live), _i32(tail_cu)
     tile, key = np.zeros(max_blocks + 1, np.int32), np.zeros(max_blocks + 1, np.int32)
     split = np.zeros(max_blocks, np.int32)
-    nb, nt, ns = C.c_int32(), C.c_int32(), C.c_int32()
-    _check(_lib.kvm_plan_attention(len(L), _p32(L), _p32(cu), int(n_q_heads), int(n_kv_heads), int(max_blocks),
-                                   C.byref(nb), C.byref(nt), _p32(tile), _p32(key), C.byref(ns), _p32(split)))
+    nw, nb, nt, ns = C.c_int32(), C.c_int32(), C.c_int32(), C.c_int32()
+    head = (len(L), _p32(L), _p32(cu), int(n_q_heads), int(n_kv_heads), int(max_blocks))
+    rest = (C.byref(nb), C.byref(nt), _p32(tile), _p32(key), C.byref(ns), _p32(split))
+    _check(_lib.kvm_plan_attention_launch(*head, C.byref(nw), *rest) if launch else _lib.kvm_plan_attention(*head, *rest))
     n = nb.value
-    return {"n_blocks": n, "n_tiles": nt.value, "block_tile": tile[:n + 1].copy(), "block_key": key[:n + 1].copy(),
+    plan = {"n_blocks": n, "n_tiles": nt.value, "block_tile": tile[:n + 1].copy(), "block_key": key[:n + 1].copy(),
             "split_first_block": split[:ns.value].copy()}
+    return dict(plan, n_waves=nw.value) if launch else plan
 
 
 def round_cost(live_after_removal, tails):

@@ -2,8 +2,10 @@
 
 kvm_plan_removal runs the span checks and the per-character bookkeeping of
 kvm_kv_compact (Eq. 2); it is compared with the oracle's span validation and
-keep mask.  kvm_plan_attention returns the attention's work partition (Eq. 3
-over the compacted cache plus the tail); it is checked against what any
+keep mask.  kvm_plan_attention returns the attention's work, cut evenly (Eq. 3
+over the compacted cache plus the tail), kvm_plan_attention_launch the
+partition that a layer runs (whole tiles dealt in waves before the cut; a block
+a tile for short caches); both are checked against what any
 correct partition must satisfy: every (query tile, key tile) unit is
 processed by exactly one block, in order, and the tiles shared by several
 blocks are listed once each with the first block that starts inside them.
@@ -180,6 +182,87 @@ def test_plan_attention_npc_round():
     plan = _check_partition([7782], [256], 16, 2, 152)
     assert plan["n_tiles"] == 32 and plan["n_blocks"] == 152
     assert len(plan["split_first_block"]) == 32
+
+
+def _check_launch_plan(live, tails, Hq, Hkv, max_blocks):
+    """Returns (waves, the block-a-tile form taken)."""
+    cu = np.concatenate([[0], np.cumsum(tails)])
+    plan = kvm.plan_attention_launch(live, cu, Hq, Hkv, max_blocks)
+    nk = _units(live, tails, Hq, Hkv)
+    G, T, W = plan["n_blocks"], plan["n_tiles"], plan["n_waves"]
+    tile, key = plan["block_tile"], plan["block_key"]
+    assert T == len(nk) and 1 <= G <= max_blocks and len(tile) == len(key) == G + 1
+    # the segments of every block as the kernel walks them: a whole tile of each
+    # wave, then the range; units [k0, k1) of a tile, and who shares a tile
+    done = [[] for _ in range(T)]
+    cost = np.zeros(G)
+    for c in range(G):
+        for w in range(W):
+            t = w * G + (G - 1 - c if w & 1 else c)
+            assert t < T
+            done[t].append((0, nk[t], c, None))
+            cost[c] += nk[t] + 8
+        (t0, k0), (t1, k1) = (tile[c], key[c]), (tile[c + 1], key[c + 1])
+        assert (t0, k0) <= (t1, k1) and t0 >= min(W * G, T) and (t1 == T and k1 == 0 or k1 < nk[t1])
+        for t in range(t0, t1 + (1 if k1 > 0 else 0)):
+            a, b = k0 if t == t0 else 0, k1 if t == t1 else nk[t]
+            assert a < b
+            # a partial's slot: the first segment of the range, or its last
+            done[t].append((a, b, c, 0 if t == t0 else 1))
+            cost[c] += b - a + 8
+            assert t in (t0, t1 if k1 > 0 else t1 - 1) or (a, b) == (0, nk[t])
+    splits = []
+    for t, parts in enumerate(done):
+        parts.sort()
+        assert [p[0] for p in parts] == [0] + [p[1] for p in parts[:-1]] and parts[-1][1] == nk[t]   # once each, in order
+        if len(parts) > 1:
+            assert [p[2] for p in parts] == list(range(parts[0][2], parts[0][2] + len(parts)))   # neighbouring blocks
+            assert all(p[3] == 0 for p in parts[1:])              # where the merge looks for them
+            splits.append(parts[1][2])
+    assert sorted(plan["split_first_block"].tolist()) == splits
+    whole = T <= max_blocks and max(nk) <= 5
+    if whole:
+        assert (G, W, splits) == (T, 0, [])
+    else:
+        assert G == max(1, min(max_blocks, sum(nk) // 4))
+        assert W == 0 or G == max_blocks and T - W * G >= G // 2
+        # no block above its even share by more than two segments and a unit
+        assert cost.max() <= cost.sum() / G + 2 * 8 + 1
+    return W, whole
+
+
+def test_launched_plan_covers_every_unit_once():
+    rng = np.random.default_rng(300)
+    seen = {"waves": 0, "odd": 0, "whole": 0, "cut": 0, "stopped": 0}
+    for trial in range(400):
+        kind = trial % 4
+        B = int(rng.integers(1, 49))
+        top = [20000, 2000, 200, 30000][kind]
+        live = [int(rng.integers(0, top)) for _ in range(B)]
+        tails = [int(rng.integers(0, [600, 600, 20, 1024][kind])) if rng.random() > 0.1 else 0 for _ in range(B)]
+        if kind == 3:                                   # one long character among short ones
+            live = [live[0] + 5000] + [int(rng.integers(0, 40)) for _ in range(B - 1)]
+        if sum(tails) == 0:
+            tails[0] = 1
+        Hq, Hkv = [(16, 2), (8, 2), (8, 8), (32, 4)][int(rng.integers(4))]
+        G = int(rng.choice([1, 7, 152, 320]))
+        W, whole = _check_launch_plan(live, tails, Hq, Hkv, G)
+        tiles = len(_units(live, tails, Hq, Hkv))
+        seen["waves"] += W > 0
+        seen["odd"] += W > 1
+        seen["whole"] += whole
+        seen["cut"] += W == 0 and not whole
+        seen["stopped"] += not whole and tiles - W * G >= G + G // 2        # too uneven for another wave
+    assert min(seen.values()) >= 5, seen
+
+
+@pytest.mark.parametrize("nk,waves,whole", [(5, 0, True), (6, 0, False)])
+def test_launched_plan_at_the_short_caches_limit(nk, waves, whole):
+    """A block a tile up to 5 key tiles (and as many tiles as blocks)."""
+    live = [64 * nk - 16]
+    assert _check_launch_plan(live, [16], 16, 2, 152) == (waves, whole)
+    assert _check_launch_plan(live * 76, [16] * 76, 16, 2, 152) == (waves, whole)
+    assert _check_launch_plan(live * 77, [16] * 77, 16, 2, 152)[1] is False       # 154 tiles
 
 
 def test_plan_attention_rejects_bad_shapes():
