@@ -763,7 +763,9 @@ __global__ void __launch_bounds__(kPrepThreads, PER_SM) gdn_prep_kernel(const __
     gdn_prep_run<DK, PER_SM>(p, FuseCtl{nullptr, 0}, blockIdx.x, gridDim.x);
 }
 
-// v2 prep: the front (loads .. [W | U]) is the v1 prep's; the record differs.
+// v2 prep: the front (loads .. [W | U]) computes what the v1 prep's does, in
+// PrepWide's layout (a block an SM, L and the inverses in rows of their own); the
+// record differs.
 template <int DK>
 __device__ __forceinline__ void gdn_prep2_run(const GdnParams& p, const FuseCtl& fc, int u0, int ustride) {
     using G = PrepWide<DK>;
@@ -1287,7 +1289,7 @@ struct ScanCfg {
 // 79.5 -> 77.7; the rest is the MMAs and the records' way from DRAM, 144 KB a
 // chunk and head.
 template <int DK, int CW, int NH>
-__device__ __forceinline__ void gdn_scan_run(const GdnParams& p, const FuseCtl& fc, int b, int h, int r0) {
+__device__ __forceinline__ void gdn_scan_run(const GdnParams& p, int b, int h, int r0) {
     using G = ScanCfg<DK>;
     using R = Rec<DK>;
     extern __shared__ uint8_t smem_raw[];
@@ -1367,13 +1369,9 @@ __device__ __forceinline__ void gdn_scan_run(const GdnParams& p, const FuseCtl& 
     // The state slice comes from an earlier round (or kvm_set_state), which
     // completed before the prep kernel this launch follows had started, so
     // it is staged before waiting for that kernel; its records are not.
-    if (!fc.flags) {                                 // the fused kernel waited already
-        grid_dependency_wait();
-        grid_dependents_launch();
-    }
-    // fused: the first record must have been published (a failed wait
-    // raises the abort flag, which stops the block at its first MMA wait)
-    if (tid == 0 && wait_record(fc, (int64_t)ch.chunk_off * H + h, &abort_flag, p.err, p.diag, 0x5f)) {
+    grid_dependency_wait();
+    grid_dependents_launch();
+    if (tid == 0) {
         mbar_arrive_expect_tx(bar_wq, G::WQ);
         bulk_load(sb + G::OFF_WQ, rec_of(0), G::WQ, bar_wq);
         mbar_arrive_expect_tx(bar_k, G::KI);
@@ -1405,8 +1403,6 @@ __device__ __forceinline__ void gdn_scan_run(const GdnParams& p, const FuseCtl& 
         const int64_t tok0 = ch.tail_off + (int64_t)i * C;
         const uint8_t* rec = rec_of(i);
         const float* misc = reinterpret_cast<const float*>(rec + R::misc_off(dv));
-        // L2-coherent loads: in a fused launch the record was written by
-        // another block of this grid
         const float wt = __ldcg(misc + (row & 63));
         const float gC = __ldcg(misc + C);
         // ---------------------------------------------------------------- [W; Q'] S0^T
@@ -1432,10 +1428,7 @@ __device__ __forceinline__ void gdn_scan_run(const GdnParams& p, const FuseCtl& 
         }
         ok = mma_wait();
         if (!ok) break;
-        // [W;Q'] image consumed: fetch the next one (fused: once the prep
-        // has published that record; a failed wait raises the abort flag)
-        if (tid == 0 && i + 1 < nch &&
-            wait_record(fc, (int64_t)(ch.chunk_off + i + 1) * H + h, &abort_flag, p.err, p.diag, 0x5e + 256 * i)) {
+        if (tid == 0 && i + 1 < nch) {                  // [W;Q'] image consumed: fetch the next one
             mbar_arrive_expect_tx(bar_wq, G::WQ);
             bulk_load(sb + G::OFF_WQ, rec_of(i + 1), G::WQ, bar_wq);
         }
@@ -1821,7 +1814,7 @@ __device__ __forceinline__ void gdn_scan_packed_run(const GdnParams& p, const Fu
 template <int DK, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? 512 : kThreads, 1) gdn_scan_kernel(const __grid_constant__ GdnParams p) {
     const int b = p.order[blockIdx.z];
-    if constexpr (WIDE) gdn_scan_run<DK, 16, 4>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
+    if constexpr (WIDE) gdn_scan_run<DK, 16, 4>(p, b, blockIdx.y, blockIdx.x * p.dv_slice);
     else gdn_scan_packed_run<DK>(p, FuseCtl{nullptr, 0}, b, blockIdx.y, blockIdx.x * p.dv_slice);
 }
 
@@ -1838,7 +1831,7 @@ __global__ void __launch_bounds__(WIDE ? 512 : kThreads, 1) gdn_scan_kernel(cons
 // cooperative launch: that one waited for every SM to be free, and so for
 // the compaction blocks beside it (a round 6.56 against 6.46 ms).
 // ============================================================================
-template <int DK, int CW>
+template <int DK>
 __global__ void __launch_bounds__(kPrepThreads, 1) gdn_fused_kernel(const __grid_constant__ GdnParams p) {
     // each role waits for the previous grid after its own set-up (below)
     const FuseCtl fc{p.flags, p.epoch};
@@ -2251,7 +2244,7 @@ void launch_scan_dk(const GdnParams& p, cudaStream_t s) {
 template <int DK>
 cudaError_t launch_fused_dk(const GdnParams& p, int grid, cudaStream_t s) {
     constexpr int smem = std::max(ScanCfg<DK>::SMEM, PrepCfg<DK, 1>::SMEM + 1024);
-    configure_once<gdn_fused_kernel<DK, 16>>(smem);
+    configure_once<gdn_fused_kernel<DK>>(smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kPrepThreads);
@@ -2262,7 +2255,7 @@ cudaError_t launch_fused_dk(const GdnParams& p, int grid, cudaStream_t s) {
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gdn_fused_kernel<DK, 16>, p);
+    return cudaLaunchKernelEx(&cfg, gdn_fused_kernel<DK>, p);
 }
 
 template <int DK>
