@@ -22,12 +22,13 @@
 // workspace; row blocks that do not fit together are done in turn).  8192 keys,
 // 8 queries of 16 heads of 256 (0.54 GFLOP): rotate 4, scores 18,
 // rows 5, probs 5 us alone, 48 together, against 210 with the scores formed
-// twice by 128 threads a tile and one thread a row merging the tiles
+// twice by 128 threads a tile and one thread a row merging the tiles.
 // Fp32 products throughout: on the tensor cores the queries would have to be
 // split, and this is the reference that other paths are judged by.
 #include <algorithm>
 
 #include "kvm_internal.cuh"
+#include "packed_f32.cuh"
 
 namespace kvm {
 namespace {
@@ -37,24 +38,6 @@ constexpr int kScoreThreads = 128;
 constexpr int kDims = 32;                      // dims staged per step
 constexpr int kPitch = 64 + 4;                 // row pitch of the staged [dim][64] tiles
 constexpr int kProbThreads = 256;              // probe_probs: 32 keys, eight threads each
-
-using f2 = unsigned long long;                 // two packed floats
-
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
 
 // One block per (query, head).
 __global__ void __launch_bounds__(128) probe_rotate_kernel(const __grid_constant__ ProbeParams p) {
