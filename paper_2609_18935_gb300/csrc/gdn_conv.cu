@@ -14,7 +14,8 @@
 // consecutive packed tokens with the taps and the last three inputs in
 // registers, four rows in flight; a head's d_k / 8 neighbouring lanes share
 // the norm of k.  Strips are as long as the grid allows: a strip's first
-// three rows are read again.
+// three rows are read again.  8674 tokens of 6144 channels (213 MB): 60 us, 3.6
+// TB/s, against 417 with a block a token and head; the exact SiLU is 7 of it.
 //
 // blockIdx.y < n_strips: outputs of a strip; beyond: one row of blocks per
 // character writes the character's new state (the last three inputs of

@@ -1279,12 +1279,13 @@ kvm_status do_gdn(kvm_ctx* c, int layer, const int32_t* tail_cu, const void* q, 
     const bool chain = c->gdn_chain && c->gdn_snap && dv_slice == 32;   // the state-chain form, where it is switched on
     const bool recur = longest <= recur_tail(c->dk) && !chain && !on_gates &&
                        (c->conv || !(on_q || on_k || on_v));
-    // its blocks each convolve their head's q and k themselves: cheaper than a
-    // launch for a few tokens (one character's decode step 4.0 against 4.4 us,
-    // 32 characters' 15.6 against 16.4; at 4 tokens 6.4 : 7.5 and 25 : 21)
     // inputs of the convolution may lie off the 16-byte grid (its own launch reads
     // them channel by channel then)
     const bool aligned = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
+    // a step's blocks each convolve their head's q and k themselves: cheaper than a
+    // launch for a few tokens (16 heads of 128, back to back: a decode step of one
+    // character 2.8 against 4.3 us, of 32 characters 10.7 : 13.8; 4 tokens of one
+    // character 4.0 : 5.8, of eight 7.0 : 8.5, of 32 25 : 21)
     const bool conv_inside = c->conv && recur && aligned && !(on_q || on_k || on_v || out == v) &&
                              (longest <= 2 || (longest <= 4 && total <= 32));
     if (c->conv && !conv_inside) {

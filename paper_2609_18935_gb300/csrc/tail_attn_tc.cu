@@ -9,8 +9,9 @@
 // neighbouring blocks at the same time, from its first key on, and share its
 // K/V through L2.  With contiguous ranges alone each block streamed the keys
 // again for every tile of its range: 32 characters' 544 MB of K/V cost 9.2 GB of
-// DRAM reads (2.9 now) and the layer 1340 us (1015 now), a 16896-token prefill
-// 1790 us (1660 now).
+// DRAM reads against 2.9, the layer 1340 us against 1015, a 16896-token prefill
+// 1790 against 1660 (both sides before the softmax groups below; 1000 - 1030 and
+// 1630 with them).
 // The rest is cut into contiguous ranges, one per block (stream-K), balanced by a
 // cost model that charges each unit 1 and each segment a block starts 8 more (the
 // host planner bisects for the smallest per-block cost).  A block's range covers whole
@@ -50,8 +51,9 @@
 // buffer, which a thread with a whole row empties at once.  With each row split
 // between two warps, two S buffers and P in shared memory (the same barriers a
 // unit, both warps in lockstep) a layer of 1024 tokens at 32K took 370 us against
-// 349, the population's 1036 : 1010, a 16896-token prefill 1651 : 1621.  Long
-// attention runs at the power limit (SM clock 1.7 - 1.9 GHz).
+// 349, the population's 1036 : 1010, a 16896-token prefill 1651 : 1621 (tiles dealt
+// on both sides, same box).  Long attention runs at the power limit (SM clock 1.7 -
+// 1.9 GHz).
 // Q lives in TMEM rather than shared memory: S_j then reads only K_j from
 // shared memory, and the space goes to a third K and V stage.
 // Every mbarrier wait is bounded in time.  On expiry the block raises an
