@@ -269,7 +269,7 @@ kvm_status kvm_tail_attn_prefill(kvm_ctx* ctx, int32_t layer, const int32_t* tai
  *   o_t = S_t q_t,
  * computed in chunks of 64 tokens (WY/UT form) starting at the first tail
  * token, or token by token when no character has more than 32 (d_k 64: 48)
- * and out, unless it is v itself, does not overlie the inputs.
+ * and out does not overlie what that form reads beside its outputs.
  * S is updated in place in the context.  out may overlie any of the inputs:
  * they are read before an output takes their place.
  * q, k device [sum M][n_gdn_heads][d_k] bf16 (k expected unit-norm per head
